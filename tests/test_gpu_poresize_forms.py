@@ -1,0 +1,23 @@
+"""The pore-size kernels at the sizes where their packing can go wrong, against
+the oracle: boxes whose edges are one below, at and above the 32-bit words and
+the 4-voxel bricks they work on, edges of one voxel, and masks so full that
+lines run through many words or close on themselves.  Counts are integers and
+the sizes fixed sequences of double operations, so the comparison is exact."""
+import numpy as np
+import pytest
+
+import synthetic as S
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(33, 32, 31), (31, 33, 65), (64, 1, 7), (3, 7, 1), (1, 40, 33), (34, 63, 97), (5, 6, 129)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("p", [0.5, 0.97, 0.9995, 1.0])
+def test_chord13_words_and_loops(orc, om, shape, p):
+    mask = S.random_mask(shape, p, 11)
+    d_o, w_o = orc.chord13(mask, 1.5, counts=True)
+    d, w = om.om_local_pore_diameter(mask, om.domain(shape, 1.5), om.OM_PORE_CHORD13, witness=True)
+    assert np.array_equal(w, w_o)
+    assert np.array_equal(d, d_o)
