@@ -21,3 +21,15 @@ def test_chord13_words_and_loops(orc, om, shape, p):
     d, w = om.om_local_pore_diameter(mask, om.domain(shape, 1.5), om.OM_PORE_CHORD13, witness=True)
     assert np.array_equal(w, w_o)
     assert np.array_equal(d, d_o)
+
+
+# small boxes: the oracle tests every pair of voxels
+@pytest.mark.parametrize("shape", [(64, 1, 7), (3, 7, 1), (1, 40, 33), (5, 6, 129), (9, 5, 4), (17, 13, 19), (21, 15, 18)])
+@pytest.mark.parametrize("p", [0.5, 0.97, 0.9995])
+def test_inscribed_bricks(orc, om, shape, p):
+    mask = S.random_mask(shape, p, 12)
+    mask.flat[mask.size // 2] = 0
+    rc, d_o, r2_o = orc.mis(mask, 1.5)
+    d, r2 = om.om_local_pore_diameter(mask, om.domain(shape, 1.5), om.OM_PORE_MIS, witness=True)
+    assert rc == 0 and np.array_equal(r2, r2_o)
+    assert np.array_equal(d, d_o)
