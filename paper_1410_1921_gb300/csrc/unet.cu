@@ -440,34 +440,39 @@ om_status conv_tc(const om_unet* U, const bf16* x1, int c1, int ld1, int o1, con
   if (N % 16 || N < 16 || N > 256 || c1 < 8 || (c1 % 8) || (c2 % 8) || (ld1 % 8) || (o1 % 8) || (ldy % 8) || (oy % 8))
     return fail(OM_EINVAL, "U-Net: convolution shape outside the tensor-core kernel's layout");
   CUtensorMap m1, m2, mw;
-  if (c2 == 0 && c1 <= 32 && (N <= 64 || !yf)) {
-    // resident weights: one persistent CTA per SM (conv3d_tc_res); wider outputs in parts
-    // of at most 64 channels (multiples of 16), one launch each
-    OM_TRY(activation_map(&m1, x1, c1, ld1, o1, g, 1));
-    const int nparts = (N + 63) / 64, width = ((N + nparts - 1) / nparts + 15) / 16 * 16;
+  const int nch = (c1 + 31) / 32 + (c2 + 31) / 32;
+  if (nch <= 3 && !yf) {
+    // planes marched with the weights of np output channels resident (conv3d_tc_zm): equal parts of
+    // N, multiples of 16, as wide as 3 np <= 256 columns and the shared memory beside nch + 1 halo
+    // buffers allow
+    constexpr size_t kSmem = 227 * 1024 - 1280;  // static shared memory set aside
+    int np = 0;
+    for (int d = 5; d >= 1 && !np; --d)
+      if ((N / 16) % d == 0 && zm_smem(nch + 1, nch, 16 * d) <= kSmem) np = 16 * d;
+    if ((c2 > 0 && ((ld2 % 8) || (o2 % 8)))) return fail(OM_EINVAL, "U-Net: second input not 16-byte aligned");
+    OM_TRY(activation_map(&m1, x1, c1, ld1, o1, g, 2));
+    if (c2 > 0) OM_TRY(activation_map(&m2, x2, c2, ld2, o2, g, 2));
+    else m2 = m1;
+    OM_TRY(weight_map(&mw, wt, c1 + c2, N, true, np));
     int dev = 0, sms = 0;
     OM_CUDA(cudaGetDevice(&dev));
     OM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    for (int n0 = 0; n0 < N; n0 += width) {
-      const int np = std::min(width, N - n0);
-      OM_TRY(weight_map(&mw, wt, c1, N, true, np));
-      TcConvArgs a{};
-      a.c1 = c1, a.c2 = 0, a.N = np, a.bias = bias ? bias + n0 : nullptr, a.y = y, a.ldy = ldy, a.oy = oy + n0;
-      a.yf = yf, a.relu = relu, a.g = g, a.nw = N, a.n0 = n0;
-      a.tx = (g.W + kTcTx - 1) / kTcTx, a.ty = (g.H + kTcTy - 1) / kTcTy;
-      a.err = U->tc_err.p;
-      const int64_t tiles = (int64_t)g.B * g.D * a.ty * a.tx;
-      // as many halo buffers (2..4) as 227 KB of shared memory hold next to the weights, and
-      // as many accumulators (2..4) as 256 TMEM columns
-      auto smem_for = [&](int nh) { return 1024 + (size_t)nh * kTrHalo + 27 * (size_t)np * 64 + 8 * 18 + 16; };
-      a.nhalo = 4;
-      while (a.nhalo > 2 && smem_for(a.nhalo) > 227 * 1024) --a.nhalo;
-      a.nacc = std::min(4, 256 / np);
-      const size_t smem = smem_for(a.nhalo);
-      OM_CUDA(cudaFuncSetAttribute(conv3d_tc_res, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      conv3d_tc_res<<<(unsigned)std::min<int64_t>(tiles, sms), kTrThreads, smem, s>>>(m1, mw, a);
-      OM_CUDA(cudaGetLastError());
-    }
+    TcConvArgs a{};
+    a.c1 = c1, a.c2 = c2, a.N = np, a.bias = bias, a.y = y, a.ldy = ldy, a.oy = oy, a.relu = relu, a.g = g;
+    a.nw = N, a.npart = N / np;
+    a.tx = (g.W + kTcTx - 1) / kTcTx, a.ty = (g.H + kTcTy - 1) / kTcTy;
+    a.err = U->tc_err.p;
+    a.nhalo = nch + 1;
+    while (a.nhalo < kZmMaxHalo && zm_smem(a.nhalo + 1, nch, np) <= kSmem) ++a.nhalo;
+    a.nacc = std::min(kZmMaxRing, 512 / np);
+    const size_t smem = zm_smem(a.nhalo, nch, np);
+    // one CTA per SM; each part's CTAs share the planes of all columns
+    const int64_t planes = (int64_t)g.B * a.ty * a.tx * g.D;
+    const unsigned grid = (unsigned)(a.npart * std::min<int64_t>(planes, std::max(1, sms / a.npart)));
+    auto k = nch == 1 ? (c1 <= 16 ? conv3d_tc_zm<1, 1> : conv3d_tc_zm<1, 2>) : (nch == 2 ? conv3d_tc_zm<2, 2> : conv3d_tc_zm<3, 2>);
+    OM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k<<<grid, kZmThreads, smem, s>>>(m1, m2, mw, a);
+    OM_CUDA(cudaGetLastError());
     return OM_OK;
   }
   OM_TRY(activation_map(&m1, x1, c1, ld1, o1, g));

@@ -10,9 +10,10 @@
 //   forward    Y[v][n] = sum_k sum_c X[v + o_k][c] WT[k][n][c]
 //   data grad  the forward kernels on dY with WT[k][ci][co] = W[26-k][ci][co]
 //   weight grad  dW[k][ci][co] = sum_v X[v + o_k][ci] dY[v][co]
-// Kernels: conv3d_tc (below), conv3d_tc_res (the forward with resident
-// weights, for narrow inputs), conv3d_wgrad_tc and conv3d_wgrad_tc32 (the
-// weight gradient; the second for at most 32 output channels).
+// Kernels: conv3d_tc (below), conv3d_tc_zm (inputs of up to 96 channels:
+// resident weights, one plane at a time), conv3d_wgrad_tc and
+// conv3d_wgrad_tc32 (the weight gradient; the second for at most 32 output
+// channels).
 //
 // conv3d_tc: implicit GEMM  Y[v][n] = sum_k sum_c X[v + o_k][c] WT[k][n][c]  with a CTA
 // tile of M = 128 voxels (a box of 8 x 8 x 2 voxels in x, y, z) and all N
@@ -60,7 +61,7 @@ constexpr int kTcStages = 3;
 constexpr int kTcThreads = 128;
 constexpr uint32_t kTcATile = kTcM * kTcKc * 2;  // 16 KB
 constexpr unsigned long long kTcSpin = 1ull << 26;  // try_wait rounds before giving up
-// the resident-weight form's tile (8 x 16 voxels at one z) and its halo box
+// the plane-marching form's and the weight gradient's tile (8 x 16 voxels at one z) and its halo box
 constexpr int kTcTx = 8, kTcTy = 16;
 constexpr int kTcHx = kTcTx + 2, kTcHy = kTcTy + 2, kTcHz = 3;
 constexpr int kTcHRows = kTcHx * kTcHy * kTcHz;  // 540 rows
@@ -74,9 +75,10 @@ struct TcConvArgs {
   float* yf;          // optional FP32 copy, rows of N
   int relu;
   Grid g;
-  int tx, ty, tz;     // tiles along x, y, z (8, 8, 2 voxels each; the resident form: 8, 16, 1)
-  int nhalo, nacc;    // the resident form's halo buffers and TMEM accumulators (2..4 each)
-  int nw, n0;         // the resident form: weight rows per offset in WT, and this launch's first
+  int tx, ty, tz;     // tiles along x, y, z (8, 8, 2 voxels each; the plane-marching form: 8, 16)
+  // the plane-marching form: N is one part's output channels, of npart parts
+  int nhalo, nacc;    // its halo buffers and the planes of its accumulator ring
+  int nw, npart;      // weight rows per offset in WT (all parts), parts
   int* err;           // set when a wait ran out
 };
 
@@ -140,6 +142,51 @@ __host__ __device__ constexpr uint32_t tc_idesc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// One MMA / one commit, issued by one lane of a converged warp (`lead`: elect_lane(), taken once).
+// The whole warp runs the issuing loop, its warp index taken through a shuffle, and the
+// instruction is predicated instead of branched around: then the compiler keeps descriptors in
+// uniform registers, where the instruction wants them, and only their low words change.  Under a
+// single thread's branch, with 64-bit descriptor arithmetic, issuing cost 70 to 110 clocks per MMA,
+// more than most of these MMAs take.
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t lead;
+  asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(lead));
+  return lead;
+}
+// descriptors as (low word, high word): the start-address field lies in the low word
+__device__ __forceinline__ void mma_f16(uint32_t lead, uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                        uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p, q;\n.reg .b64 a, b;\nsetp.ne.b32 q, %0, 0;\nsetp.ne.b32 p, %7, 0;\n"
+      "mov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%1], a, b, %6, p;\n}" ::"r"(lead),
+      "r"(d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t lead, uint32_t bar) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %0, 0;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n}" ::"r"(lead),
+      "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ uint32_t lo32(uint64_t v) { return (uint32_t)v; }
+__device__ __forceinline__ uint32_t hi32(uint64_t v) { return (uint32_t)(v >> 32); }
+// mbar_wait by a whole warp with one answer for all its lanes
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const volatile int* stop) {
+  uint32_t now;
+  asm volatile(
+      "{\n.reg .pred p;\n"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(now)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  if (__all_sync(0xffffffffu, now)) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, stop)) != 0;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ CUtensorMap map1,
                                                         const __grid_constant__ CUtensorMap map2,
                                                         const __grid_constant__ CUtensorMap mapw, TcConvArgs a) {
@@ -155,7 +202,7 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ 
   __shared__ volatile int stop;         // a wait ran out: issue nothing more
   __shared__ int n_issued, n_consumed;  // copies issued / waited for by the MMA thread
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8u * kTcStages, done = full0 + 16u * kTcStages;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
 
   // tile coordinates
   int t = blockIdx.x;
@@ -218,34 +265,25 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ 
     }
     n_issued = s;
     if (s < nsteps) stop = 1;
-  } else if (tid == 32) {
+  } else if (warp == 1) {
     // MMA issue: four K = 16 slices per stage, accumulating in TMEM
-    const uint32_t idesc = tc_idesc(kTcM, a.N);
+    const uint32_t idesc = tc_idesc(kTcM, a.N), lead = elect_lane(), dhi = hi32(sw128_desc(0u));
     int s = 0;
     for (; s < nsteps; ++s) {
       const int st = s % kTcStages;
-      if (!mbar_wait(full0 + 8u * st, (uint32_t)(s / kTcStages) & 1u, &stop)) break;
+      if (!warp_wait(full0 + 8u * st, (uint32_t)(s / kTcStages) & 1u, &stop)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t sa = base + (uint32_t)st * stage_bytes, sb = sa + kTcATile;
+      const uint32_t alo = lo32(sw128_desc(sa)), blo = lo32(sw128_desc(sb));
 #pragma unroll
-      for (int kk = 0; kk < kTcKc / 16; ++kk) {
-        const uint64_t ad = sw128_desc(sa + 32u * kk), bd = sw128_desc(sb + 32u * kk);
-        const uint32_t acc = (s > 0 || kk > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-            : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       empty0 + 8u * st)
-                   : "memory");
+      for (int kk = 0; kk < kTcKc / 16; ++kk)
+        mma_f16(lead, tmem, alo + 2u * kk, dhi, blo + 2u * kk, dhi, idesc, (s > 0 || kk > 0) ? 1u : 0u);
+      mma_commit(lead, empty0 + 8u * st);
     }
     n_consumed = s;
     if (s < nsteps) stop = 1;
     // `done` fires when every MMA issued above has completed
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
-                 : "memory");
+    mma_commit(lead, done);
   }
   const bool fin = mbar_wait(done, 0);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -305,63 +343,89 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
 }
 
-// ------------------------------------------------------------------ resident-weight form
-// For a single input of at most 32 channels and at most 64 output channels
-// (the finest level's convolutions, which carry most of the voxels) the
-// whole operand WT[27][N][32] fits in shared memory next to two halo
-// buffers: a persistent CTA per SM loads the weights once and then walks its
-// tiles (8 x 16 voxels at one z).  Per tile TMA copies the halo -- 10 x 18 x
-// 3 voxels of 32 channels, rows of 64 bytes with the 64-byte swizzle -- and
-// the 27 filter offsets read it through shifted descriptors (the swizzle is
-// applied to the absolute shared-memory address, so a view shifted by whole
-// rows inside the TMA-written box is consistent).  Warp 0 issues the copies,
-// warp 1 the MMAs (2 per offset, K = 16) into one of two TMEM accumulators,
-// warps 2-5 drain the other accumulator (bias, ReLU, BF16 store) while the
-// next tile accumulates.  Channels past the input's count are the copy's
-// zero fill.  nhalo halo buffers and nacc accumulators (2..4 each, as the
-// shared memory and TMEM allow) keep that many tiles in flight.  Waits are
-// bounded as in conv3d_tc.
-constexpr int kTrThreads = 192;
-constexpr uint32_t kTrHBox = (uint32_t)kTcHRows * 64u;        // 34560 bytes
-constexpr uint32_t kTrHalo = (kTrHBox + 1023u) / 1024u * 1024u;  // 34816
+// ------------------------------------------------------------------ plane-marching form
+// conv3d_tc_zm: inputs of up to 96 channels (three chunks of 32).  A CTA keeps the weights of `np`
+// output channels resident and walks the z planes of an 8 x 16-voxel column.  One input plane
+// contributes to three output planes, through the filter's dz = +1, 0, -1 parts, so the three
+// output planes' accumulators sit side by side in TMEM and the weight rows of the three parts side
+// by side in shared memory: one MMA of N = 3 np does what three of N = np did, on one read of its A
+// operand, and a plane's halo (10 x 18 voxels, rows of 64 bytes, 64-byte swizzle) is copied once
+// instead of three times.  With N = 32 the shared-memory reads of A (4 KB per 128 x 32 x 16 MMA)
+// and the issue of 54 small MMAs a tile set the pace (the form before this one, three planes of halo
+// per tile: 20 % tensor-pipe activity).  Measured (4 x 64^3; K in, N out channels): 16 -> 32 from
+// 110 to 50 us, 32 -> 32 110 to 65, 96 -> 32 (then on conv3d_tc) 448 to 160, 64 -> 64 at 32^3 51 to 33.
+// What is left above the MMAs' own ~56 clocks each is the issuing warp's work between planes
+// (~1200 clocks: waits, commits, ring bookkeeping).
+//
+// The accumulators form a ring of R planes in TMEM: input plane z adds to planes z - 1, z, z + 1
+// (two MMAs where the ring wraps), plane z - 1 is then complete and drained by warps 2-5 (bias,
+// ReLU, BF16 store) while the next planes accumulate.  Planes outside the box are skipped: they
+// are zeros.  Every output sums its products in the order of conv3d_tc: filter offsets k = 0..26,
+// per offset the channels upwards.
+//
+// Warp 0 issues the copies (weights once, then 32-channel planes into a ring of nhalo buffers),
+// warp 1 the MMAs.  CTA i of a part (blockIdx.x % npart) takes an equal share of the planes of all
+// columns laid end to end; a share that starts inside a column reads up to two planes more than it
+// puts out.  Waits are bounded as in conv3d_tc.
+constexpr int kZmThreads = 192;
+constexpr int kZmMaxRing = 32, kZmMaxHalo = 12;
+constexpr uint32_t kZmBox = (uint32_t)(kTcHx * kTcHy) * 64u;      // 11520 bytes
+constexpr uint32_t kZmBuf = (kZmBox + 1023u) / 1024u * 1024u;     // 12288
+constexpr uint32_t kZmBars = 8u * (2 * kZmMaxHalo + 2 * kZmMaxRing + 2) + 16u;
 
 __device__ __forceinline__ uint64_t sw64_desc(uint32_t addr, uint32_t sbo) {
   return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
-__global__ void __launch_bounds__(kTrThreads) conv3d_tc_res(const __grid_constant__ CUtensorMap map1,
-                                                            const __grid_constant__ CUtensorMap mapw, TcConvArgs a) {
+// shared memory of a launch: alignment slack, halo buffers, weights, barriers
+__host__ __device__ constexpr size_t zm_smem(int nhalo, int nch, int np) {
+  return 1024 + (size_t)nhalo * kZmBuf + (size_t)27 * nch * np * 64 + kZmBars;
+}
+
+// NCH: 32-channel chunks of the input(s); KK: K = 16 slices of a chunk (1: one input of 16 channels)
+template <int NCH, int KK>
+__global__ void __launch_bounds__(kZmThreads) conv3d_tc_zm(const __grid_constant__ CUtensorMap map1,
+                                                           const __grid_constant__ CUtensorMap map2,
+                                                           const __grid_constant__ CUtensorMap mapw, TcConvArgs a) {
   extern __shared__ uint8_t tc_smem_raw[];
-  // [halo x nhalo][weights 27 x N rows x 64 B][barriers][TMEM address], 1024-byte aligned
   const uint32_t raw = smem_u32(tc_smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = tc_smem_raw + (base - raw);
-  const int NH = a.nhalo, NA = a.nacc;
-  const uint32_t wbox = (uint32_t)a.N * 64u, wres = base + (uint32_t)NH * kTrHalo;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + (size_t)NH * kTrHalo + 27 * (size_t)wbox);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
-  const uint32_t b0 = smem_u32(bars);
-  const uint32_t wfull = b0, hfull0 = b0 + 8u, hempty0 = b0 + 40u, afull0 = b0 + 72u, aempty0 = b0 + 104u,
-                 done = b0 + 136u;
+  const int NH = a.nhalo, R = a.nacc;
+  const uint32_t np = (uint32_t)a.N;                                    // output channels of this CTA
+  const uint32_t wres = base + (uint32_t)NH * kZmBuf, brow = np * 64u;  // weights; bytes of one part's rows
+  uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + (size_t)NH * kZmBuf + (size_t)27 * NCH * brow);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kZmMaxHalo + 2 * kZmMaxRing + 2);
+  const uint32_t wfull = smem_u32(bars), done = wfull + 8u, hfull0 = done + 8u, hempty0 = hfull0 + 8u * kZmMaxHalo,
+                 afull0 = hempty0 + 8u * kZmMaxHalo, aempty0 = afull0 + 8u * kZmMaxRing;
   __shared__ volatile int stop;
   __shared__ int h_issued, h_used;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ntiles = a.g.B * a.g.D * a.ty * a.tx;
-  uint32_t ncols = 32u;  // NA accumulators of N columns, a power of two
-  while (ncols < (uint32_t)(NA * a.N)) ncols <<= 1;
+  __shared__ __align__(16) float sbias[256];
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int D = a.g.D, n1 = (a.c1 + 31) / 32;
+  const int part = (int)blockIdx.x % a.npart, n0 = part * a.N;
+  // this CTA's planes of all columns laid end to end
+  const int64_t planes = (int64_t)a.g.B * a.ty * a.tx * D;
+  const int64_t share = blockIdx.x / a.npart, shares = gridDim.x / a.npart;
+  const int64_t lo = planes * share / shares, hi = planes * (share + 1) / shares;
+  uint32_t ncols = 32u;
+  while (ncols < (uint32_t)R * np) ncols <<= 1;
 
+  for (int i = tid; i < (int)np; i += kZmThreads) sbias[i] = a.bias ? a.bias[n0 + i] : 0.f;
   if (tid == 0) {
     stop = 0;
     h_issued = h_used = 0;
     mbar_init(wfull, 1);
-    for (int i = 0; i < 4; ++i) {
+    mbar_init(done, 1);
+    for (int i = 0; i < NH; ++i) {
       mbar_init(hfull0 + 8u * i, 1);
       mbar_init(hempty0 + 8u * i, 1);
+    }
+    for (int i = 0; i < R; ++i) {
       mbar_init(afull0 + 8u * i, 1);
       mbar_init(aempty0 + 8u * i, 4);  // one arrival per epilogue warp
     }
-    mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -376,128 +440,212 @@ __global__ void __launch_bounds__(kTrThreads) conv3d_tc_res(const __grid_constan
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
-  auto tile_xyz = [&](int t, int& x0, int& y0, int& z0, int& bb) {
-    x0 = (t % a.tx) * kTcTx;
-    t /= a.tx;
-    y0 = (t % a.ty) * kTcTy;
-    t /= a.ty;
-    z0 = t % a.g.D;
-    bb = t / a.g.D;
+  // a run of planes [zs, ze) of one column starting at plane p of the whole
+  struct Run {
+    int x0, y0, bb, zs, ze;
+  };
+  auto run_at = [&](int64_t p) {
+    Run r;
+    int64_t c = p / D;
+    r.zs = (int)(p - c * D);
+    r.ze = (int)min((int64_t)D, r.zs + (hi - p));
+    r.x0 = (int)(c % a.tx) * kTcTx;
+    c /= a.tx;
+    r.y0 = (int)(c % a.ty) * kTcTy;
+    r.bb = (int)(c / a.ty);
+    return r;
   };
 
   if (tid == 0) {
-    // producer: the weights once, then each tile's halo into the buffer its
-    // tile two back has released
-    mbar_expect_tx(wfull, 27u * wbox);
-    for (int k = 0; k < 27; ++k) tma_load_2d(wres + (uint32_t)k * wbox, &mapw, 0, k * a.nw + a.n0, wfull);
-    int i = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
-      const int hb = i % NH;
-      if (i >= NH && !mbar_wait(hempty0 + 8u * hb, (uint32_t)(i / NH - 1) & 1u, &stop)) break;
-      if (stop) break;
-      int x0, y0, z0, bb;
-      tile_xyz(t, x0, y0, z0, bb);
-      mbar_expect_tx(hfull0 + 8u * hb, kTrHBox);
-      tma_load_5d(base + (uint32_t)hb * kTrHalo, &map1, 0, x0 - 1, y0 - 1, z0 - 1, bb, hfull0 + 8u * hb);
-      h_issued = i + 1;
+    // producer: the weights, rows of the parts dz = +1, 0, -1 of each (dy, dx) and chunk together
+    mbar_expect_tx(wfull, 27u * NCH * brow);
+    for (int k9 = 0; k9 < 9; ++k9)
+      for (int c = 0; c < NCH; ++c)
+        for (int d = 0; d < 3; ++d)
+          tma_load_2d(wres + (uint32_t)((k9 * NCH + c) * 3 + d) * brow, &mapw, c < n1 ? 32 * c : a.c1 + 32 * (c - n1),
+                      ((2 - d) * 9 + k9) * a.nw + n0, wfull);
+    int i = 0, hb = 0;
+    uint32_t lap = 1u;  // parity of the release that frees buffer hb; the first lap waits for none
+    bool ok = true;
+    for (int64_t p = lo; ok && p < hi;) {
+      const Run r = run_at(p);
+      const int zl = min(r.ze, D - 1);
+      for (int z = max(r.zs - 1, 0); ok && z <= zl; ++z)
+        for (int c = 0; c < NCH; ++c) {
+          if (i >= NH && !mbar_wait(hempty0 + 8u * hb, lap, &stop)) ok = false;
+          if (stop) ok = false;
+          if (!ok) break;
+          mbar_expect_tx(hfull0 + 8u * hb, kZmBox);
+          tma_load_5d(base + (uint32_t)hb * kZmBuf, c < n1 ? &map1 : &map2, c < n1 ? 32 * c : 32 * (c - n1), r.x0 - 1,
+                      r.y0 - 1, z, r.bb, hfull0 + 8u * hb);
+          h_issued = ++i;
+          if (++hb == NH) {
+            hb = 0;
+            lap ^= 1u;
+          }
+        }
+      p += r.ze - r.zs;
     }
-    if (blockIdx.x + (int64_t)h_issued * gridDim.x < ntiles) stop = 1;
-  } else if (tid == 32) {
-    // MMA issue
-    const uint32_t idesc = tc_idesc(kTcM, a.N);
-    bool ok = mbar_wait(wfull, 0, &stop);
-    int i = 0;
-    for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x, ++i) {
-      const int hb = i % NH, ab = i % NA;
-      if (i >= NA && !mbar_wait(aempty0 + 8u * ab, (uint32_t)(i / NA - 1) & 1u, &stop)) break;
-      if (!mbar_wait(hfull0 + 8u * hb, (uint32_t)(i / NH) & 1u, &stop)) break;
-      h_used = i + 1;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t hbase = base + (uint32_t)hb * kTrHalo, acc_addr = tmem + (uint32_t)(ab * a.N);
-      // descriptors of offset k, slice kk: the start-address field (address / 16)
-      // of the first ones advanced by the offset's row shift and the slice's 32 bytes
-      const uint64_t ad0 = sw64_desc(hbase, kTcHx * 64u), bd0 = sw64_desc(wres, 512u);
-      const uint64_t bstep = wbox >> 4;
+    if (!ok) stop = 1;
+  } else if (warp == 1) {
+    // MMA issue.  Ring positions advance by counting, not by division: this warp's instructions between
+    // two MMAs are time the tensor pipe may wait for.
+    const uint32_t idesc1 = tc_idesc(kTcM, (int)np) - ((np >> 3) << 17);  // without N
+    const uint32_t lead = elect_lane();
+    bool ok = warp_wait(wfull, 0, &stop);
+    int used = 0;                  // planes of 32 channels taken
+    int hb = 0;                    // the next one's buffer
+    uint32_t hlap = 0u;            // and the parity of its lap
+    int nslot = 0, cslot = 0;      // ring slots of the next plane to start and the next to complete
+    uint32_t nlap = 1u;            // parity of the drain that frees nslot; the first lap waits for none
+    bool lap0 = true;
+    for (int64_t p = lo; ok && p < hi;) {
+      const Run r = run_at(p);
+      const int zl = min(r.ze, D - 1);
+      int olo = r.zs, slo = nslot;  // first output plane this input adds to, and its slot
+      for (int z = max(r.zs - 1, 0); z <= zl; ++z) {
+        if (z - 1 > olo) {
+          ++olo;
+          if (++slo == R) slo = 0;
+        }
+        const int ohi = min(z + 1, r.ze - 1), onew = max(olo, z == 0 ? 0 : z + 1);
+        for (int o = onew; o <= ohi; ++o) {  // a slot is free again once drained
+          if (!lap0) ok = ok && warp_wait(aempty0 + 8u * nslot, nlap, &stop);
+          if (++nslot == R) {
+            nslot = 0;
+            nlap ^= 1u;
+            lap0 = false;
+          }
+        }
+        if (!ok) break;
+        uint32_t alo[NCH], hbar[NCH], hpar[NCH];
 #pragma unroll
-      for (int k = 0; k < 27; ++k) {
-        constexpr uint32_t kRow = 64u / 16u;  // a halo row in units of 16 bytes
-        const uint32_t shift = (uint32_t)((((k / 9) * kTcHy) + (k / 3) % 3) * kTcHx + k % 3) * kRow;
+        for (int c = 0; c < NCH; ++c) {
+          alo[c] = lo32(sw64_desc(base + (uint32_t)hb * kZmBuf, 0u));
+          hbar[c] = 8u * hb;
+          hpar[c] = hlap;
+          if (++hb == NH) {
+            hb = 0;
+            hlap ^= 1u;
+          }
+        }
+        const uint32_t ahi = hi32(sw64_desc(0u, kTcHx * 64u)), bhi = hi32(sw64_desc(0u, 512u));
+        const int cnt = ohi - olo + 1, first = min(cnt, R - slo);  // planes before the ring wraps
+        for (int w = 0; w < 2; ++w) {
+          const int plo = w ? olo + first : olo, pn = w ? cnt - first : first;
+          if (pn <= 0) break;
+          const uint32_t dcol = tmem + (uint32_t)(w ? 0 : slo) * np;
+          const uint32_t idesc = idesc1 + (((uint32_t)pn * np >> 3) << 17);
+          uint32_t blo = lo32(sw64_desc(wres + (uint32_t)(plo - (z - 1)) * brow, 0u));
+          const uint32_t bstep = 3u * brow >> 4;
+          const int old = min(max(onew - plo, 0), pn);  // planes that already hold sums
+          constexpr uint32_t kRow = 64u / 16u;          // a halo row in units of 16 bytes
 #pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-          const uint64_t ad = ad0 + shift + 2u * kk;
-          const uint64_t bd = bd0 + (uint64_t)k * bstep + 2u * kk;
-          const uint32_t acc = (k > 0 || kk > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(acc_addr),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-              : "memory");
+          for (int k9 = 0; k9 < 9; ++k9) {
+            const uint32_t shift = (uint32_t)((k9 / 3) * kTcHx + k9 % 3) * kRow;
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+              if (k9 == 0) {
+                if (w == 0) {  // the chunk's first use
+                  ok = ok && warp_wait(hfull0 + hbar[c], hpar[c], &stop);
+                  if (!ok) break;
+                  h_used = ++used;
+                  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
+                if (c == 0 && old < pn) {
+                  // the first product of the planes that start here overwrites their slots
+                  if (old > 0)
+                    mma_f16(lead, dcol, alo[0], ahi, blo, bhi, idesc1 + (((uint32_t)old * np >> 3) << 17), 1u);
+                  mma_f16(lead, dcol + (uint32_t)old * np, alo[0], ahi, blo + (uint32_t)old * (brow >> 4), bhi,
+                          idesc1 + (((uint32_t)(pn - old) * np >> 3) << 17), 0u);
+                } else {
+                  mma_f16(lead, dcol, alo[c], ahi, blo, bhi, idesc, 1u);
+                }
+              } else {
+                mma_f16(lead, dcol, alo[c] + shift, ahi, blo, bhi, idesc, 1u);
+              }
+              if (KK > 1) mma_f16(lead, dcol, alo[c] + shift + 2u, ahi, blo + 2u, bhi, idesc, 1u);
+              blo += bstep;
+            }
+            if (k9 == 0 && !ok) break;
+          }
+          if (!ok) break;
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) mma_commit(lead, hempty0 + hbar[c]);
+        // planes complete after this one: z - 1, and z itself at the far face
+        if (z - 1 >= r.zs) {
+          mma_commit(lead, afull0 + 8u * cslot);
+          if (++cslot == R) cslot = 0;
+        }
+        if (z == D - 1 && z < r.ze) {
+          mma_commit(lead, afull0 + 8u * cslot);
+          if (++cslot == R) cslot = 0;
         }
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       hempty0 + 8u * hb)
-                   : "memory");
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       afull0 + 8u * ab)
-                   : "memory");
+      p += r.ze - r.zs;
     }
-    if (!ok || blockIdx.x + (int64_t)h_used * gridDim.x < ntiles) stop = 1;
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
-                 : "memory");
+    if (!ok) stop = 1;
+    mma_commit(lead, done);
   } else if (warp >= 2) {
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows
-    const int q = warp & 3, r = q * 32 + lane;
-    int i = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
-      const int ab = i % NA;
-      if (!mbar_wait(afull0 + 8u * ab, (uint32_t)(i / NA) & 1u, &stop)) {
-        if (lane == 0) stop = 1;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      int x0, y0, z0, bb;
-      tile_xyz(t, x0, y0, z0, bb);
-      const int xx = x0 + (r & 7), yy = y0 + (r >> 3);
+    const int qd = warp & 3, rr = qd * 32 + lane;
+    int slot = 0;
+    uint32_t lap = 0u;
+    bool ok = true;
+    for (int64_t p = lo; ok && p < hi;) {
+      const Run r = run_at(p);
+      const int xx = r.x0 + (rr & 7), yy = r.y0 + (rr >> 3);
       const bool inside = xx < a.g.W && yy < a.g.H;
-      const int64_t v = inside ? (((int64_t)bb * a.g.D + z0) * a.g.H + yy) * a.g.W + xx : 0;
-      for (int c0 = 0; c0 < a.N; c0 += 16) {
-        uint32_t qv[16];
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * a.N + c0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15}, [%16];"
-            : "=r"(qv[0]), "=r"(qv[1]), "=r"(qv[2]), "=r"(qv[3]), "=r"(qv[4]), "=r"(qv[5]), "=r"(qv[6]),
-              "=r"(qv[7]), "=r"(qv[8]), "=r"(qv[9]), "=r"(qv[10]), "=r"(qv[11]), "=r"(qv[12]), "=r"(qv[13]),
-              "=r"(qv[14]), "=r"(qv[15])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (!inside) continue;
-        float f[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          f[j] = __uint_as_float(qv[j]) + (a.bias ? a.bias[c0 + j] : 0.f);
-          if (a.relu) f[j] = fmaxf(f[j], 0.f);
+      const int64_t plane = (int64_t)a.g.H * a.g.W * a.ldy;
+      bf16* dst = inside ? a.y + ((((int64_t)r.bb * D + r.zs) * a.g.H + yy) * a.g.W + xx) * a.ldy + a.oy + n0 : a.y;
+      for (int z = r.zs; z < r.ze; ++z, dst += plane) {
+        if (!warp_wait(afull0 + 8u * slot, lap, &stop)) {
+          if (lane == 0) stop = 1;
+          ok = false;
+          break;
         }
-        if (a.y) {
-          uint32_t p[8];
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int c0 = 0; c0 < (int)np; c0 += 16) {
+          uint32_t qv[16];
+          const uint32_t taddr = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)slot * np + (uint32_t)c0;
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+              "%14, %15}, [%16];"
+              : "=r"(qv[0]), "=r"(qv[1]), "=r"(qv[2]), "=r"(qv[3]), "=r"(qv[4]), "=r"(qv[5]), "=r"(qv[6]),
+                "=r"(qv[7]), "=r"(qv[8]), "=r"(qv[9]), "=r"(qv[10]), "=r"(qv[11]), "=r"(qv[12]), "=r"(qv[13]),
+                "=r"(qv[14]), "=r"(qv[15])
+              : "r"(taddr));
+          float bias[16];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 b = *reinterpret_cast<const float4*>(&sbias[c0 + 4 * j]);
+            bias[4 * j] = b.x, bias[4 * j + 1] = b.y, bias[4 * j + 2] = b.z, bias[4 * j + 3] = b.w;
+          }
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (!inside) continue;
+          uint32_t o[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * j], f[2 * j + 1]);
-            p[j] = *reinterpret_cast<const uint32_t*>(&h);
+            float f0 = __uint_as_float(qv[2 * j]) + bias[2 * j], f1 = __uint_as_float(qv[2 * j + 1]) + bias[2 * j + 1];
+            if (a.relu) f0 = fmaxf(f0, 0.f), f1 = fmaxf(f1, 0.f);
+            const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
+            o[j] = *reinterpret_cast<const uint32_t*>(&h);
           }
-          uint4* dst = reinterpret_cast<uint4*>(a.y + v * a.ldy + a.oy + c0);
-          dst[0] = make_uint4(p[0], p[1], p[2], p[3]);
-          dst[1] = make_uint4(p[4], p[5], p[6], p[7]);
+          uint4* d4 = reinterpret_cast<uint4*>(dst + c0);
+          d4[0] = make_uint4(o[0], o[1], o[2], o[3]);
+          d4[1] = make_uint4(o[4], o[5], o[6], o[7]);
         }
-        if (a.yf) {
-          float4* dst = reinterpret_cast<float4*>(a.yf + v * a.N + c0);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) dst[j] = make_float4(f[4 * j], f[4 * j + 1], f[4 * j + 2], f[4 * j + 3]);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty0 + 8u * slot) : "memory");
+        if (++slot == R) {
+          slot = 0;
+          lap ^= 1u;
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty0 + 8u * ab) : "memory");
+      p += r.ze - r.zs;
     }
   }
   const bool fin = mbar_wait(done, 0);
@@ -518,7 +666,7 @@ __global__ void __launch_bounds__(kTrThreads) conv3d_tc_res(const __grid_constan
 // dW[k][ci][co] = sum over voxels v of X[v + o_k][ci] dY[v][co], read in
 // place: no transposed copies.  Both operands are "MN-major" (channels
 // contiguous, voxels along K) views of TMA copies with the 64-byte swizzle:
-// A of the input's halo (rows of 32 channels, as conv3d_tc_res loads it), B
+// A of the input's halo (rows of 32 channels, as conv3d_tc_zm loads it), B
 // of the 8 x 16-voxel tile of dY (one 32-channel atom per 8 KB).  An MN atom
 // of A is 32 channels; its four atoms sit one halo row (64 bytes) apart, so
 // one MMA's 128 rows of D are the channels of the offsets dx = -1, 0, +1 (and
@@ -543,6 +691,7 @@ struct TcWgradArgs {
   int* err;
 };
 
+constexpr uint32_t kTrHalo = ((uint32_t)kTcHRows * 64u + 1023u) / 1024u * 1024u;  // three planes of the halo
 constexpr uint32_t kWgPlane = (uint32_t)(kTcHx * kTcHy) * 64u;  // 11520: one z plane of the halo
 constexpr uint32_t kWgAtom = 128u * 64u;                         // 8192: 32 channels of the dY tile
 
@@ -573,7 +722,7 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8u * S, done = full0 + 16u * S;
   __shared__ volatile int stop;
   __shared__ int n_issued, n_used;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int ntiles = a.g.B * a.g.D * a.ty * a.tx;
   // this CTA's input chunk and (dz, dy) group
   const int ngroup = 9 / a.npair;
@@ -634,13 +783,13 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
       n_issued = i + 1;
     }
     if (i < mytiles) stop = 1;
-  } else if (tid == 32) {
+  } else if (warp == 1) {
     // MMA issue: per pair and two y rows, A = halo rows (plane, y + dy, x + dx) for dx = 0..3
-    const uint32_t idesc = tc_idesc(kTcM, a.Nm) | (1u << 15) | (1u << 16);
+    const uint32_t idesc = tc_idesc(kTcM, a.Nm) | (1u << 15) | (1u << 16), lead = elect_lane();
     int i = 0;
     for (; i < mytiles; ++i) {
       const int st = i % S;
-      if (!mbar_wait(full0 + 8u * st, (uint32_t)(i / S) & 1u, &stop)) break;
+      if (!warp_wait(full0 + 8u * st, (uint32_t)(i / S) & 1u, &stop)) break;
       n_used = i + 1;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t sa = base + (uint32_t)st * stage_bytes;
@@ -649,25 +798,17 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
         const int pr = pair0 + p, dz = pr / 3, dy = pr % 3;
         const uint32_t row = (uint32_t)((a.npair == 9 ? dz * kTcHy : 0) + dy) * kTcHx;  // first halo row
         const uint32_t acc_addr = tmem + (uint32_t)(p * a.Nm);
+        const uint32_t alo = lo32(ad0) + row * 4u;  // 64-byte rows in units of 16 bytes
+        const uint32_t acc = i > 0 ? 1u : 0u;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint64_t ad = ad0 + (row + (uint32_t)kk * 2u * kTcHx) * 4u;  // 64-byte rows in units of 16 bytes
-          const uint64_t bd = bd0 + (uint32_t)kk * 64u;                      // 1024 bytes: two rows of 8 voxels
-          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(acc_addr),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-              : "memory");
-        }
+        for (int kk = 0; kk < 8; ++kk)  // two y rows: 2 halo rows of A, 1024 bytes of B
+          mma_f16(lead, acc_addr, alo + (uint32_t)kk * 8u * kTcHx, hi32(ad0), lo32(bd0) + (uint32_t)kk * 64u, hi32(bd0),
+                  idesc, kk > 0 ? 1u : acc);
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       empty0 + 8u * st)
-                   : "memory");
+      mma_commit(lead, empty0 + 8u * st);
     }
     if (i < mytiles) stop = 1;
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
-                 : "memory");
+    mma_commit(lead, done);
   }
   const bool fin = mbar_wait(done, 0);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -742,7 +883,7 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc32(const __grid_con
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8u * S, done = full0 + 16u * S;
   __shared__ volatile int stop;
   __shared__ int n_issued, n_used;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int tyx = a.ty + 1;  // tile rows, the last one two rows high
   const int ntiles = a.g.B * a.g.D * tyx * a.tx;
   const int chunk = (int)blockIdx.y;
@@ -796,12 +937,12 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc32(const __grid_con
       n_issued = i + 1;
     }
     if (i < mytiles) stop = 1;
-  } else if (tid == 32) {
-    const uint32_t idesc = tc_idesc(kTcM, 96) | (1u << 15) | (1u << 16);
+  } else if (warp == 1) {
+    const uint32_t idesc = tc_idesc(kTcM, 96) | (1u << 15) | (1u << 16), lead = elect_lane();
     int i = 0;
     for (; i < mytiles; ++i) {
       const int st = i % S;
-      if (!mbar_wait(full0 + 8u * st, (uint32_t)(i / S) & 1u, &stop)) break;
+      if (!warp_wait(full0 + 8u * st, (uint32_t)(i / S) & 1u, &stop)) break;
       n_used = i + 1;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int yt = (blockIdx.x + i * gridDim.x) / a.tx % tyx;
@@ -810,26 +951,21 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc32(const __grid_con
       // A: dY, atoms one tile row (512 bytes) apart, K-groups one tile row apart;
       // B: the planes, atoms one halo row (64 bytes) apart, K-groups 10 rows apart
       const uint64_t ad0 = mn_sw64_desc(sa + kWnB, 512u, 512u), bd0 = mn_sw64_desc(sa, 64u, kTcHx * 64u);
+      const uint32_t acc = i > 0 ? 1u : 0u;
+#pragma unroll
       for (int dz = 0; dz < 3; ++dz) {
-        const uint32_t acc_addr = tmem + (uint32_t)(dz * 96);
-        for (int kk = 0; kk < nk; ++kk) {
-          const uint64_t ad = ad0 + (uint32_t)kk * 64u;                                    // 1024 bytes
-          const uint64_t bd = bd0 + ((uint32_t)dz * 160u + (uint32_t)kk * 2u * kTcHx) * 4u;  // 64-byte rows
-          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(acc_addr),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-              : "memory");
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+          if (kk > 0 && kk >= nk) break;
+          // A 1024 bytes a K = 16 step; B 64-byte rows, two halo rows a step
+          mma_f16(lead, tmem + (uint32_t)(dz * 96), lo32(ad0) + (uint32_t)kk * 64u, hi32(ad0),
+                  lo32(bd0) + ((uint32_t)dz * 160u + (uint32_t)kk * 2u * kTcHx) * 4u, hi32(bd0), idesc, kk > 0 ? 1u : acc);
         }
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       empty0 + 8u * st)
-                   : "memory");
+      mma_commit(lead, empty0 + 8u * st);
     }
     if (i < mytiles) stop = 1;
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
-                 : "memory");
+    mma_commit(lead, done);
   }
   const bool fin = mbar_wait(done, 0);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
