@@ -292,17 +292,13 @@ __global__ void __launch_bounds__(kTile) flow_batch_observe(FlowArgs<T> a, const
       if (ODD) flow_neighbours(b, b.coord[ln], nb);
       C f[19];
       flow_load<T, ODD>(b, n, nb, f);
-      double rho = 0, jx = 0;
-#pragma unroll
-      for (int i = 0; i < 19; ++i) {
-        rho += (double)f[i];
-        jx += (double)q19_e(i, 0) * (double)f[i];
-      }
-      const double ux = jx + 0.5 * (double)a.g;
+      double m[2];
+      wide_sums<SumMassX19>(f, m);
+      const double ux = m[1] + 0.5 * (double)a.g;
       acc[0] = ux;
       acc[1] = fabs(ux - prev[n]);
       acc[2] = fabs(ux);
-      acc[3] = rho + flow_ref(a, n);
+      acc[3] = m[0] + flow_ref(a, n);
       prev[n] = ux;
     }
     block_reduce_write<4>(acc, partials + (int64_t)w * 4);
@@ -336,12 +332,11 @@ __global__ void __launch_bounds__(kTile) diff_batch_observe(DiffArgs<T> a, const
       if (ODD) diff_neighbours(b, b.coord[ln], nb, x);
       C g[7];
       diff_load<T, D3Q7, ODD>(b, n, nb, x, g);
-      double dev = 0;
-#pragma unroll
-      for (int i = 0; i < 7; ++i) dev += (double)g[i];
-      const double c = dev + diff_ref(b, n, x);
+      double m[2];
+      wide_sums<SumMassX<D3Q7>>(g, m);
+      const double c = m[0] + diff_ref(b, n, x);
       const double om = (double)b.omega[n];
-      acc[0] = (1.0 - 0.5 * om) * ((double)g[1] - (double)g[2]);
+      acc[0] = (1.0 - 0.5 * om) * m[1];
       acc[1] = fabs(c - prev[n]);
       acc[2] = fabs(c);
       acc[3] = c;
@@ -422,10 +417,9 @@ __global__ void flow_batch_export(FlowArgs<T> a, uint32_t off, const int64_t* vo
     for (int i = 0; i < 19; ++i) out[i * N + v] = (double)f[i] + q19_w(i) * r1;
   }
   if (ux) {
-    double jx = 0.0;
-#pragma unroll
-    for (int i = 0; i < 19; ++i) jx += (double)q19_e(i, 0) * (double)f[i];
-    ux[v] = (float)(jx + 0.5 * (double)a.g);
+    double j[1];
+    wide_sums<SumX19>(f, j);
+    ux[v] = (float)(j[0] + 0.5 * (double)a.g);
   }
 }
 
@@ -443,13 +437,15 @@ __global__ void diff_batch_export(DiffArgs<T> a, uint32_t off, const int64_t* vo
   diff_load<T, D3Q7, ODD>(a, off + ln, nb, x, g);
   const int64_t v = vox[ln];
   const double cref = diff_ref(a, off + ln, x);
-  double dev = 0.0;
+  if (out) {
 #pragma unroll
-  for (int i = 0; i < 7; ++i) {
-    dev += (double)g[i];
-    if (out) out[i * N + v] = (double)g[i] + q7_w(i) * cref;
+    for (int i = 0; i < 7; ++i) out[i * N + v] = (double)g[i] + q7_w(i) * cref;
   }
-  if (c) c[v] = (float)(dev + cref);
+  if (c) {
+    double m[2];
+    wide_sums<SumMassX<D3Q7>>(g, m);
+    c[v] = (float)(m[0] + cref);
+  }
 }
 
 template <class T>
@@ -491,11 +487,7 @@ __global__ void flow_batch_init(FlowArgs<T> a, uint32_t off, const int64_t* vox,
   if (ln >= a.nf) return;
   const double u = warm_velocity(scale * (double)field[vox[ln] * stride]);
   if constexpr (kFlowRebased<T>) a.rr[off + ln] = 0.f;
-#pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    const double eu = (double)q19_e(i, 0) * u;
-    Stg<T>::st(a.s[i] + off + ln, (typename Stg<T>::C)(q19_w(i) * (3.0 * eu + 4.5 * eu * eu - 1.5 * u * u)), a.up);
-  }
+  flow_store_eq_x(a, off + ln, u);
 }
 
 template <class T>
@@ -514,7 +506,10 @@ __global__ void diff_batch_init(DiffArgs<T> a, uint32_t off, const int64_t* vox,
     dc = 0.0;
   }
 #pragma unroll
-  for (int i = 0; i < 7; ++i) Stg<T>::st(a.q[i] + off + ln, (typename Stg<T>::C)(q7_w(i) * dc), a.up);
+  for (int i = 0; i < 7; ++i) {
+    if constexpr (kRebased<T>) Stg<T>::st(a.q[i] + off + ln, 0, a.up);
+    else Stg<T>::st(a.q[i] + off + ln, (typename Stg<T>::C)(q7_w(i) * dc), a.up);
+  }
 }
 
 // 16-bit diffusion: reference of every node of every structure set to C_lin(x)

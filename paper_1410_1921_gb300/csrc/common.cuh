@@ -110,8 +110,16 @@ __host__ __device__ inline void unpack_xyz(uint32_t c, int& x, int& y, int& z) {
 }
 
 // ------------------------------------------------------------------ misc
-constexpr int kObsBlocks = 1216;  // 8 x 152 SMs: fixed grid of reductions
+// fixed grid of reductions: 5 x 152 SMs, the blocks of the D3Q19 observables (48 registers) that are
+// resident at once (8 x 152 left a second, half-empty wave; more and smaller blocks spend FP64
+// operations on their reductions)
+constexpr int kObsBlocks = 760;
 constexpr int kObsThreads = 256;
+// blocks of a reduction over nf nodes: the fixed grid, or as many as have nodes
+inline int obs_blocks(uint32_t nf) {
+  const int64_t b = ((int64_t)nf + kObsThreads - 1) / kObsThreads;
+  return b < 1 ? 1 : (b < kObsBlocks ? (int)b : kObsBlocks);
+}
 
 // Blocks of `threads` threads of `kernel` (with `smem` bytes of dynamic
 // shared memory) that fit on the device at once (SMs x resident blocks per

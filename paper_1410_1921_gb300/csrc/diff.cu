@@ -121,8 +121,9 @@ __global__ void __launch_bounds__(256) diff_sweep_pair(DiffArgs<T, L> a) {
   else diff_pair_even<T, L>(a, n);
 }
 
-// Observables: sum J_x, sum |C - prev|, sum |C|, sum C, sum D_L; prev <- C.
-template <class T, class L, bool ODD>
+// Observables: sum J_x, sum |C - prev|, sum |C|, sum C, sum D_L (DL: only
+// where the caller reads it; it costs a double division per node); prev <- C.
+template <class T, class L, bool ODD, bool DL>
 __global__ void __launch_bounds__(kObsThreads) diff_observe(DiffArgs<T, L> a, double* prev,
                                                             double* partials, double* dprev) {
   using C = typename Stg<T>::C;
@@ -134,20 +135,16 @@ __global__ void __launch_bounds__(kObsThreads) diff_observe(DiffArgs<T, L> a, do
     if (ODD) diff_neighbours(a, a.coord[n], nb, x);
     C g[L::Q];
     diff_load<T, L, ODD>(a, n, nb, x, g);
-    double dev = 0, ex = 0;
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      dev += (double)g[i];
-      if (L::e(i, 0)) ex += L::e(i, 0) > 0 ? (double)g[i] : -(double)g[i];
-    }
-    const double c = dev + diff_ref(a, n, x);
+    double m[2];
+    wide_sums<SumMassX<L>>(g, m);
+    const double c = m[0] + diff_ref(a, n, x);
     const double om = (double)a.omega[n];
-    const double jx = (1.0 - 0.5 * om) * ex;
+    const double jx = (1.0 - 0.5 * om) * m[1];
     acc[0] += jx;
     acc[1] += fabs(c - prev[n]);
     acc[2] += fabs(c);
     acc[3] += c;
-    acc[4] += L::cs2 * (1.0 / om - 0.5);
+    if constexpr (DL) acc[4] += L::cs2 * (1.0 / om - 0.5);
     if (dprev) dprev[n] = c - prev[n];
     prev[n] = c;
   }
@@ -191,15 +188,16 @@ __global__ void diff_export(DiffArgs<T, L> a, const int64_t* vox, int64_t N, dou
   diff_load<T, L, ODD>(a, n, nb, x, g);
   const int64_t v = vox[n];
   const double cref = diff_ref(a, n, x);
-  double dev = 0, ex = 0;
+  if (gdense) {
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    dev += (double)g[i];
-    if (L::e(i, 0)) ex += L::e(i, 0) > 0 ? (double)g[i] : -(double)g[i];
-    if (gdense) gdense[i * N + v] = (double)g[i] + L::w(i) * cref;
+    for (int i = 0; i < L::Q; ++i) gdense[i * N + v] = (double)g[i] + L::w(i) * cref;
   }
-  if (cdense) cdense[v] = (float)(dev + cref);
-  if (jdense) jdense[v] = (float)((1.0 - 0.5 * (double)a.omega[n]) * ex);
+  if (cdense || jdense) {
+    double m[2];
+    wide_sums<SumMassX<L>>(g, m);
+    if (cdense) cdense[v] = (float)(m[0] + cref);
+    if (jdense) jdense[v] = (float)((1.0 - 0.5 * (double)a.omega[n]) * m[1]);
+  }
 }
 
 // populations from the dense layout (linear != 0: the linear profile a_i C_lin);
@@ -223,11 +221,19 @@ __global__ void diff_import(DiffArgs<T, L> a, const int64_t* vox, int64_t N, con
     a.cr[n] = (float)ref;
     ref = (double)a.cr[n];
   }
+  if (linear) {  // one value per weight: rest, axis, diagonal
+    typename S::C w[3];
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    const double g = linear ? L::w(i) * clin : gdense[i * N + v];
-    S::st(a.q[i] + n, (typename S::C)(g - L::w(i) * ref), a.up);
+    for (int k = 0; k < 3; ++k) {
+      const double wk = L::w(k == 0 ? 0 : (k == 1 ? 1 : L::Q - 1));
+      w[k] = (typename S::C)(wk * clin - wk * ref);
+    }
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) S::st(a.q[i] + n, w[i == 0 ? 0 : (i < 7 ? 1 : 2)], a.up);
+    return;
   }
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) S::st(a.q[i] + n, (typename S::C)(gdense[i * N + v] - L::w(i) * ref), a.up);
 }
 
 // warm start: g_i = a_i C (deviation a_i (C - C_lin(x))) in the even layout
@@ -247,7 +253,10 @@ __global__ void diff_init_c(DiffArgs<T, L> a, const int64_t* vox, const float* c
     dc = cv - clin;
   }
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) Stg<T>::st(a.q[i] + n, (typename Stg<T>::C)(L::w(i) * dc), a.up);
+  for (int i = 0; i < L::Q; ++i) {
+    if constexpr (kRebased<T>) Stg<T>::st(a.q[i] + n, 0, a.up);
+    else Stg<T>::st(a.q[i] + n, (typename Stg<T>::C)(L::w(i) * dc), a.up);
+  }
 }
 
 template <class T, class L>
@@ -463,11 +472,13 @@ om_status diff_tune_t(om_diff* df, cudaStream_t s) {
 }
 
 template <class T, class L>
-om_status diff_observe_t(om_diff* df, double* out, cudaStream_t s) {
+om_status diff_observe_t(om_diff* df, double* out, bool with_dl, cudaStream_t s) {
   DiffArgs<T, L> a = diff_args<T, L>(df);
-  if (df->t & 1) diff_observe<T, L, true><<<kObsBlocks, kObsThreads, 0, s>>>(a, df->prev, df->partials, df->dprev);
-  else diff_observe<T, L, false><<<kObsBlocks, kObsThreads, 0, s>>>(a, df->prev, df->partials, df->dprev);
-  launch_finalize(df->partials, kObsBlocks, 5, df->obs_dev, s);
+  const int nblk = obs_blocks(a.nf);
+  auto k = df->t & 1 ? (with_dl ? diff_observe<T, L, true, true> : diff_observe<T, L, true, false>)
+                     : (with_dl ? diff_observe<T, L, false, true> : diff_observe<T, L, false, false>);
+  k<<<nblk, kObsThreads, 0, s>>>(a, df->prev, df->partials, df->dprev);
+  launch_finalize(df->partials, nblk, 5, df->obs_dev, s);
   OM_CUDA(cudaGetLastError());
   OM_CUDA(cudaMemcpyAsync(df->obs_host, df->obs_dev, 5 * sizeof(double), cudaMemcpyDeviceToHost, s));
   OM_CUDA(cudaStreamSynchronize(s));
@@ -560,8 +571,9 @@ om_status diff_rebase_t(om_diff* df, cudaStream_t s) {
   return OM_OK;
 }
 
-om_status diff_observe_any(om_diff* df, double* out, cudaStream_t s) {
-  OM_DIFF_DISPATCH(df, diff_observe_t, df, out, s);
+// with_dl: out[4] = sum D_L too (else 0)
+om_status diff_observe_any(om_diff* df, double* out, bool with_dl, cudaStream_t s) {
+  OM_DIFF_DISPATCH(df, diff_observe_t, df, out, with_dl, s);
 }
 
 }  // namespace
@@ -627,7 +639,7 @@ extern "C" om_status om_diff_create(const om_nodeset* ns, const float* d_nm_dev,
   }
   if (st == OM_OK) {
     double o[5];
-    st = diff_observe_any(df, o, s);
+    st = diff_observe_any(df, o, false, s);
   }
   if (st != OM_OK) {
     om_diff_destroy(df);
@@ -645,7 +657,7 @@ extern "C" om_status om_diff_step(om_diff* df, int64_t nsteps, void* stream) {
 
 extern "C" om_status om_diff_observe(om_diff* df, double* out, void* stream) {
   if (!df || !out) return fail(OM_EINVAL, "om_diff_observe: null pointer");
-  return diff_observe_any(df, out, as_stream(stream));
+  return diff_observe_any(df, out, true, as_stream(stream));
 }
 
 extern "C" om_status om_diff_solve(om_diff* df, double* D_eff_lattice, om_run_info* info,
@@ -659,7 +671,7 @@ extern "C" om_status om_diff_solve(om_diff* df, double* D_eff_lattice, om_run_in
   OM_CUDA(cudaEventCreate(&e0));
   OM_CUDA(cudaEventCreate(&e1));
   double o[5];
-  OM_TRY(diff_observe_any(df, o, s));
+  OM_TRY(diff_observe_any(df, o, false, s));
   double sj_prev = o[0];
   const int64_t t0 = df->t;
   OM_CUDA(cudaEventRecord(e0, s));
@@ -670,7 +682,7 @@ extern "C" om_status om_diff_solve(om_diff* df, double* D_eff_lattice, om_run_in
   while (df->t - t0 < p.max_steps) {
     int64_t k = std::min<int64_t>(p.check_every, p.max_steps - (df->t - t0));
     OM_TRY(om_diff_step(df, k, stream));
-    OM_TRY(diff_observe_any(df, o, s));
+    OM_TRY(diff_observe_any(df, o, false, s));
     // converged when both the concentration field and the total flux have
     // settled: C can sit at its final profile while the flux still relaxes
     if (!std::isfinite(o[0]) || !std::isfinite(o[2])) {
@@ -734,7 +746,7 @@ extern "C" om_status om_diff_set_populations(om_diff* df, const double* g_dev, v
   auto imp = [&]() -> om_status { OM_DIFF_DISPATCH(df, diff_import_t, df, g_dev, 0, s); };
   OM_TRY(imp());
   double o[5];
-  return diff_observe_any(df, o, s);
+  return diff_observe_any(df, o, false, s);
 }
 
 extern "C" om_status om_diff_init_concentration(om_diff* df, const float* c_dev, int64_t stride, int32_t from_linear,
@@ -744,7 +756,7 @@ extern "C" om_status om_diff_init_concentration(om_diff* df, const float* c_dev,
   auto init = [&]() -> om_status { OM_DIFF_DISPATCH(df, diff_init_c_t, df, c_dev, stride, from_linear, s); };
   OM_TRY(init());
   double o[5];
-  return diff_observe_any(df, o, s);
+  return diff_observe_any(df, o, false, s);
 }
 
 extern "C" om_status om_diff_time(const om_diff* df, int64_t* t) {

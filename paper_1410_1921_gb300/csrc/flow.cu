@@ -256,14 +256,10 @@ __global__ void __launch_bounds__(kObsThreads) d3q19_observe(FlowArgs<T> a, doub
     if (ODD) flow_neighbours(a, a.coord[n], nb);
     C f[19];
     flow_load<T, ODD>(a, n, nb, f);
-    double rho = 0, jx = 0;
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-      rho += (double)f[i];
-      jx += (double)q19_e(i, 0) * (double)f[i];
-    }
-    const double ux = jx + 0.5 * (double)a.g;
-    acc[3] += rho + flow_ref(a, n);
+    double m[2];
+    wide_sums<SumMassX19>(f, m);
+    const double ux = m[1] + 0.5 * (double)a.g;
+    acc[3] += m[0] + flow_ref(a, n);
     if (flow_boundary_index(a, n) >= 0) continue;  // pressure drive: velocity sums over interior layers
     acc[0] += ux;
     acc[1] += fabs(ux - prev[n]);
@@ -290,16 +286,11 @@ __global__ void d3q19_export(FlowArgs<T> a, const int64_t* vox, int64_t N, doubl
     for (int i = 0; i < 19; ++i) fdense[i * N + v] = (double)f[i] + q19_w(i) * r1;
   }
   if (udense) {
-    double jx = 0, jy = 0, jz = 0;
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-      jx += (double)q19_e(i, 0) * (double)f[i];
-      jy += (double)q19_e(i, 1) * (double)f[i];
-      jz += (double)q19_e(i, 2) * (double)f[i];
-    }
-    udense[v] = (float)(jx + 0.5 * (double)a.g);
-    udense[N + v] = (float)jy;
-    udense[2 * N + v] = (float)jz;
+    double j[3];
+    wide_sums<SumMomentum19>(f, j);
+    udense[v] = (float)(j[0] + 0.5 * (double)a.g);
+    udense[N + v] = (float)j[1];
+    udense[2 * N + v] = (float)j[2];
   }
 }
 
@@ -321,11 +312,7 @@ __global__ void d3q19_init_u(FlowArgs<T> a, const int64_t* vox, const float* ux,
   if (n >= a.nf) return;
   const double u = warm_velocity(scale * (double)ux[vox[n] * stride]);
   if constexpr (kFlowRebased<T>) a.rr[n] = 0.f;
-#pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    const double eu = (double)q19_e(i, 0) * u;
-    Stg<T>::st(a.s[i] + n, (typename Stg<T>::C)(q19_w(i) * (3.0 * eu + 4.5 * eu * eu - 1.5 * u * u)), a.up);
-  }
+  flow_store_eq_x(a, n, u);
 }
 
 // Pressure drive: the extrapolated pre-collision deviations of every
@@ -640,9 +627,10 @@ om_status flow_tune_t(om_flow* fl, cudaStream_t s) {
 template <class T>
 om_status flow_observe_t(om_flow* fl, double* out, cudaStream_t s) {
   FlowArgs<T> a = flow_args<T>(fl);
-  if (fl->t & 1) d3q19_observe<T, true><<<kObsBlocks, kObsThreads, 0, s>>>(a, fl->prev, fl->partials);
-  else d3q19_observe<T, false><<<kObsBlocks, kObsThreads, 0, s>>>(a, fl->prev, fl->partials);
-  launch_finalize(fl->partials, kObsBlocks, 4, fl->obs_dev, s);
+  const int nblk = obs_blocks(a.nf);
+  if (fl->t & 1) d3q19_observe<T, true><<<nblk, kObsThreads, 0, s>>>(a, fl->prev, fl->partials);
+  else d3q19_observe<T, false><<<nblk, kObsThreads, 0, s>>>(a, fl->prev, fl->partials);
+  launch_finalize(fl->partials, nblk, 4, fl->obs_dev, s);
   OM_CUDA(cudaGetLastError());
   OM_CUDA(cudaMemcpyAsync(fl->obs_host, fl->obs_dev, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
   OM_CUDA(cudaStreamSynchronize(s));

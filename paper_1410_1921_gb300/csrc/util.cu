@@ -130,20 +130,33 @@ om_status exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint6
 }
 
 // ------------------------------------------------------------------ reductions
-__global__ void finalize_partials(const double* partials, int nblk, int nval, double* out) {
-  // one block; value k summed by the block in a fixed order
-  __shared__ double sm[256];
-  for (int k = 0; k < nval; ++k) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) acc += partials[(int64_t)b * nval + k];
-    sm[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) sm[threadIdx.x] += sm[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[k] = sm[0];
-    __syncthreads();
+// one block: thread t sums its share of the blocks' partials for every value,
+// the warps reduce them together and one more warp step adds the warps' sums
+//
+constexpr int kMaxVals = 8;
+__global__ void __launch_bounds__(1024) finalize_partials(const double* partials, int nblk, int nval, double* out) {
+  __shared__ double sm[kMaxVals][32];
+  double acc[kMaxVals];
+#pragma unroll
+  for (int k = 0; k < kMaxVals; ++k) acc[k] = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
+#pragma unroll
+    for (int k = 0; k < kMaxVals; ++k)
+      if (k < nval) acc[k] += partials[(int64_t)b * nval + k];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < kMaxVals; ++k) {
+    if (k >= nval) break;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
+    if (lane == 0) sm[k][wid] = acc[k];
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < nval) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < 32; ++w) t += sm[threadIdx.x][w];
+    out[threadIdx.x] = t;
   }
 }
 
@@ -202,7 +215,7 @@ unsigned resident_blocks(const void* kernel, int threads, size_t smem) {
 }
 
 void launch_finalize(const double* partials, int nblk, int nval, double* out, cudaStream_t s) {
-  finalize_partials<<<1, 256, 0, s>>>(partials, nblk, nval, out);
+  finalize_partials<<<1, 1024, 0, s>>>(partials, nblk, nval, out);
 }
 
 }  // namespace om
