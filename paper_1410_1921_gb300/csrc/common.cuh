@@ -67,6 +67,37 @@ struct DevBuf {
   }
 };
 
+// Stream-ordered scratch of one call: allocated and freed on the stream that
+// uses it, without the device-wide wait and the mapping of a cudaMalloc /
+// cudaFree pair (calls that follow each other on a stream reuse the memory).
+struct StreamBuf {
+  void* p = nullptr;
+  cudaStream_t s;
+  explicit StreamBuf(cudaStream_t st) : s(st) {}
+  StreamBuf(const StreamBuf&) = delete;
+  StreamBuf& operator=(const StreamBuf&) = delete;
+  ~StreamBuf() {
+    if (p) cudaFreeAsync(p, s);
+  }
+  bool try_alloc(size_t bytes) {
+    if (cudaMallocAsync(&p, bytes ? bytes : 1, s) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    p = nullptr;
+    return false;
+  }
+  om_status alloc(size_t bytes) {
+    if (try_alloc(bytes)) return OM_OK;
+    return fail(OM_ENOMEM, "device scratch of " + std::to_string(bytes) + " bytes could not be allocated");
+  }
+};
+// the next part of an allocation, 256-byte aligned: *at is moved past it
+template <class T>
+inline T* carve(void* base, size_t* at, size_t count) {
+  T* q = reinterpret_cast<T*>(reinterpret_cast<char*>(base) + *at);
+  *at += (count * sizeof(T) + 255) / 256 * 256;
+  return q;
+}
+
 // ------------------------------------------------------------------ lattices
 // D3Q19 in the population order of the transformation matrix of App. A:
 // rest, +-x, +-y, +-z, then (+-1,+-1,0), (+-1,0,+-1), (0,+-1,+-1) with the
@@ -153,6 +184,7 @@ struct om_nodeset {
   int64_t N = 0;        // voxels
   int64_t nf = 0;       // nodes
   int64_t pitch = 0;    // population array stride (nodes, padded to 64)
+  void* mem = nullptr;  // the allocation that holds the arrays below
   // [nx*ny*W]: {node bits, nodes before this word, node number of the voxel
   // below the word's first and above its last (periodic in z; kNoNode if none)}
   uint4* col = nullptr;

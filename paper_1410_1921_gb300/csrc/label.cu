@@ -3,10 +3,17 @@
 // Pore voxels are joined with their 18 neighbours (the D3Q19 links; y and z
 // periodic, x not) by a lock-free union-find: a root is only ever linked
 // below a smaller index, so every component ends as a tree rooted at its
-// smallest voxel index, the canonical label.  Runs of pore voxels along z
-// start as single trees, and two runs that touch along several voxels are
-// joined once, at the lowest voxel of their overlap.  Transport voxels belong to a
+// smallest voxel index, the canonical label.  Transport voxels belong to a
 // component with voxels on both x faces.
+//
+// The nodes of the union-find are the runs of pore voxels along z, each
+// named by its first voxel.  Rows are packed to bits first; contacts between
+// neighbouring rows are then word operations, and only one union is issued
+// per pair of overlapping runs, plus the diagonal contacts that no overlap
+// implies.  256^3 at porosity 0.35: 347 us of kernels; with a tree
+// node per voxel and 27 mask reads per voxel (the form that
+// om_label_connectivity_noalloc still takes, for want of scratch for the
+// packed rows) 1430 us.
 #include <algorithm>
 
 #include "common.cuh"
@@ -112,32 +119,175 @@ __global__ void uf_flatten(int* par, int64_t N) {
     if (par[v] >= 0) par[v] = uf_root(par, (int)v);
 }
 
-__global__ void mark_faces(const int* lab, int nx, int ny, int nz, uint8_t* touch) {
-  const int64_t plane = (int64_t)ny * nz;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (int64_t)gridDim.x * blockDim.x) {
-    // flag bytes are set through their aligned 32-bit word: bit 0 inlet, bit 1 outlet
-    const int a = lab[i];
-    if (a >= 0) atomicOr((unsigned int*)(touch + (a & ~3)), 1u << (8 * (a & 3)));
-    const int b = lab[(int64_t)(nx - 1) * plane + i];
-    if (b >= 0) atomicOr((unsigned int*)(touch + (b & ~3)), 2u << (8 * (b & 3)));
+}  // namespace
+
+namespace {
+
+// Rows: bits[r * W + w], r = x * ny + y; bits past nz are zero.
+struct Rows {
+  const uint32_t* bits;
+  int nx, ny, nz, W;
+};
+
+__global__ void row_pack(const uint8_t* mask, int64_t rows, int nz, int W, uint32_t* bits) {
+  const int lane = threadIdx.x & 31;
+  const int64_t words = rows * W;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < words;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t r = i / W;
+    const int z = 32 * (int)(i - r * W) + lane;
+    const uint32_t b = __ballot_sync(0xffffffffu, z < nz && mask[r * nz + z] != 0);
+    if (lane == 0) bits[i] = b;
   }
 }
 
-__global__ void transport_from_labels(const int* lab, const uint8_t* touch, int64_t N, uint8_t* tr,
-                                      unsigned long long* counts) {
+// first voxel of the run that holds voxel z of a row
+__device__ __forceinline__ int run_head(const uint32_t* row, int z) {
+  int w = z >> 5;
+  uint32_t gap = ~__ldg(row + w) & ((1u << (z & 31)) - 1u);
+  while (!gap && w > 0) gap = ~__ldg(row + --w);
+  return gap ? 32 * w + 32 - __clz((int)gap) : 0;
+}
+
+// run heads of word w (a run does not wrap at z = 0)
+__device__ __forceinline__ uint32_t word_heads(const uint32_t* row, int w) {
+  const uint32_t b = __ldg(row + w);
+  return b & ~((b << 1) | (w > 0 ? __ldg(row + w - 1) >> 31 : 0u));
+}
+
+__global__ void run_init(Rows q, int64_t words, int* par) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / q.W;
+    const int w = (int)(i - r * q.W);
+    uint32_t h = word_heads(q.bits + r * q.W, w);
+    for (; h; h &= h - 1) {
+      const int64_t v = r * q.nz + 32 * w + __ffs((int)h) - 1;
+      par[v] = (int)v;
+    }
+  }
+}
+
+// bit z of the result: voxel z + 1 (UP) or z - 1 of the row, periodic
+template <bool UP>
+__device__ __forceinline__ uint32_t row_shift(const uint32_t* row, int w, int W, int nz) {
+  const uint32_t b = __ldg(row + w);
+  if (UP) {
+    if (w + 1 < W) return (b >> 1) | (__ldg(row + w + 1) << 31);
+    return (b >> 1) | ((__ldg(row) & 1u) << ((nz - 1) & 31));
+  }
+  if (w > 0) return (b << 1) | (__ldg(row + w - 1) >> 31);
+  return (b << 1) | ((__ldg(row + W - 1) >> ((nz - 1) & 31)) & 1u);
+}
+
+// The forward half of the 18 neighbours, one word of a row per thread.
+// Overlaps of two rows' runs (dz = 0) are joined at their first voxel;
+// contacts one voxel up or down only where neither voxel faces a pore of the
+// other row: otherwise an overlap (and a row's own join of its two ends,
+// where the contact wraps) already connects the runs.
+__global__ void run_link(Rows q, int64_t words, int* par) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / q.W;
+    const int w = (int)(i - r * q.W);
+    const uint32_t* row = q.bits + r * q.W;
+    const uint32_t a = __ldg(row + w);
+    if (!a) continue;
+    const int x = (int)(r / q.ny), y = (int)(r - (int64_t)x * q.ny);
+    const int yp = y + 1 == q.ny ? 0 : y + 1, ym = y == 0 ? q.ny - 1 : y - 1;
+    const uint32_t valid = w + 1 < q.W || (q.nz & 31) == 0 ? 0xffffffffu : (1u << (q.nz & 31)) - 1u;
+    auto join = [&](int z, int64_t r2, int z2) {
+      uf_union(par, (int)(r * q.nz) + run_head(row, z), (int)(r2 * q.nz) + run_head(q.bits + r2 * q.W, z2));
+    };
+    auto overlap = [&](int64_t r2) {
+      const uint32_t* row2 = q.bits + r2 * q.W;
+      const uint32_t c = a & __ldg(row2 + w);
+      uint32_t first = c & ~((c << 1) | (w > 0 ? (__ldg(row + w - 1) & __ldg(row2 + w - 1)) >> 31 : 0u));
+      for (; first; first &= first - 1) {
+        const int z = 32 * w + __ffs((int)first) - 1;
+        join(z, r2, z);
+      }
+    };
+    auto corners = [&](int64_t r2) {
+      const uint32_t* row2 = q.bits + r2 * q.W;
+      const uint32_t alone = a & ~__ldg(row2 + w);
+      uint32_t up = alone & row_shift<true>(row2, w, q.W, q.nz) & ~row_shift<true>(row, w, q.W, q.nz) & valid;
+      for (; up; up &= up - 1) {
+        const int z = 32 * w + __ffs((int)up) - 1;
+        join(z, r2, z + 1 == q.nz ? 0 : z + 1);
+      }
+      uint32_t dn = alone & row_shift<false>(row2, w, q.W, q.nz) & ~row_shift<false>(row, w, q.W, q.nz) & valid;
+      for (; dn; dn &= dn - 1) {
+        const int z = 32 * w + __ffs((int)dn) - 1;
+        join(z, r2, z == 0 ? q.nz - 1 : z - 1);
+      }
+    };
+    if (x + 1 < q.nx) {
+      const int64_t e = (int64_t)(x + 1) * q.ny;
+      overlap(e + y);
+      corners(e + y);
+      overlap(e + yp);
+      overlap(e + ym);
+    }
+    overlap((int64_t)x * q.ny + yp);
+    corners((int64_t)x * q.ny + yp);
+    if (w == q.W - 1 && ((a >> ((q.nz - 1) & 31)) & 1u) && (__ldg(row) & 1u)) join(q.nz - 1, r, 0);  // round the row
+  }
+}
+
+// every head to its root (no compression on the way: see uf_root), and the
+// roots of the two x faces' runs marked (bit 0 inlet, bit 1 outlet)
+__global__ void run_flatten(Rows q, int64_t words, int* par) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / q.W;
+    const int w = (int)(i - r * q.W);
+    uint32_t h = word_heads(q.bits + r * q.W, w);
+    for (; h; h &= h - 1) {
+      const int v = (int)(r * q.nz) + 32 * w + __ffs((int)h) - 1;
+      par[v] = uf_root(par, v);
+    }
+  }
+}
+
+__global__ void run_faces(Rows q, const int* par, uint8_t* touch) {
+  const int64_t face = (int64_t)q.ny * q.W;  // words of one x face
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 2 * face; i += (int64_t)gridDim.x * blockDim.x) {
+    const bool out = i >= face;
+    const int64_t k = (out ? i - face : i) / q.W, r = (out ? (int64_t)(q.nx - 1) * q.ny : 0) + k;
+    const int w = (int)((out ? i - face : i) - k * q.W);
+    uint32_t h = word_heads(q.bits + r * q.W, w);
+    for (; h; h &= h - 1) {
+      const int a = par[r * q.nz + 32 * w + __ffs((int)h) - 1];
+      atomicOr((unsigned int*)(touch + (a & ~3)), (out ? 2u : 1u) << (8 * (a & 3)));
+    }
+  }
+}
+
+// labels (LAB: in place of par, whose head entries already hold the labels),
+// transport flags and the counts, one warp per word
+template <bool LAB>
+__global__ void run_labels(Rows q, int64_t words, int* par, const uint8_t* touch, uint8_t* tr, unsigned long long* counts) {
+  const int lane = threadIdx.x & 31;
   unsigned long long np = 0, nt = 0;
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-    const int a = lab[v];
-    const bool t = a >= 0 && touch[a] == 3;
-    if (tr) tr[v] = t ? 1 : 0;
-    np += a >= 0;
-    nt += t;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < words;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t r = i / q.W;
+    const int w = (int)(i - r * q.W), z = 32 * w + lane;
+    const uint32_t* row = q.bits + r * q.W;
+    const uint32_t b = __ldg(row + w);
+    const bool pore = (b >> lane) & 1u;
+    int lab = -1;
+    bool t = false;
+    if (pore) {
+      lab = par[r * q.nz + run_head(row, z)];
+      t = touch[lab] == 3;
+    }
+    if (z < q.nz) {
+      if (LAB) par[r * q.nz + z] = lab;
+      if (tr) tr[r * q.nz + z] = t ? 1 : 0;
+    }
+    np += __popc(b);
+    nt += __popc(__ballot_sync(0xffffffffu, t));
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    np += __shfl_down_sync(0xffffffffu, np, o);
-    nt += __shfl_down_sync(0xffffffffu, nt, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
+  if (lane == 0 && np) {
     atomicAdd(counts, np);
     atomicAdd(counts + 1, nt);
   }
@@ -147,25 +297,41 @@ __global__ void transport_from_labels(const int* lab, const uint8_t* touch, int6
 
 void launch_union_find(const uint8_t* mask_dev, const om_domain& d, int* labels_dev, cudaStream_t s);
 
-// labels (int32 N) and transport flags on the device; counts of pore and
-// transport voxels returned through the host pointers when non-null.
+// labels (int32 N, nullable) and transport flags (nullable) on the device;
+// counts of pore and transport voxels returned through the host pointers
+// when non-null.
 om_status label_impl(const uint8_t* mask_dev, const om_domain& d, int* labels_dev, uint8_t* transport_dev,
                      int64_t* npore, int64_t* ntrans, cudaStream_t s) {
   const int64_t N = voxels(d);
   if (N >= (int64_t)0x7fffffff) return fail(OM_EINVAL, "labelling needs fewer than 2^31 voxels");
-  // mark_faces sets flag bytes through 32-bit words: pad to a multiple of 4
-  DevBuf<uint8_t> touch;
-  DevBuf<unsigned long long> cnt;
-  OM_TRY(touch.alloc((N + 3) / 4 * 4));
-  OM_TRY(cnt.alloc(2));
-  OM_CUDA(cudaMemsetAsync(touch.p, 0, (N + 3) / 4 * 4, s));
-  OM_CUDA(cudaMemsetAsync(cnt.p, 0, 2 * sizeof(unsigned long long), s));
-  launch_union_find(mask_dev, d, labels_dev, s);
-  mark_faces<<<152, 256, 0, s>>>(labels_dev, d.nx, d.ny, d.nz, touch.p);
-  transport_from_labels<<<1216, 256, 0, s>>>(labels_dev, touch.p, N, transport_dev, cnt.p);
+  const int W = (d.nz + 31) / 32;
+  const int64_t rows = (int64_t)d.nx * d.ny, words = rows * W;
+  // scratch: flag bytes (set through 32-bit words: padded to a multiple of 4), counters, packed rows, run parents
+  const size_t touch_bytes = (size_t)(N + 3) / 4 * 4;
+  StreamBuf buf(s);
+  size_t at = 0, need = 0;
+  for (size_t b : {touch_bytes, 2 * sizeof(unsigned long long), words * sizeof(uint32_t), labels_dev ? (size_t)0 : N * sizeof(int)})
+    need += (b + 255) / 256 * 256;
+  OM_TRY(buf.alloc(need));
+  uint8_t* touch = carve<uint8_t>(buf.p, &at, touch_bytes);
+  unsigned long long* cnt = carve<unsigned long long>(buf.p, &at, 2);
+  OM_CUDA(cudaMemsetAsync(buf.p, 0, at, s));
+  uint32_t* bits = carve<uint32_t>(buf.p, &at, words);
+  int* par = labels_dev ? labels_dev : carve<int>(buf.p, &at, N);
+  const Rows q{bits, d.nx, d.ny, d.nz, W};
+  const unsigned warps = (unsigned)std::min<int64_t>((words + 7) / 8, 16 * 1216);
+  const unsigned threads = (unsigned)std::min<int64_t>((words + 127) / 128, 16 * 1216);
+  row_pack<<<warps, 256, 0, s>>>(mask_dev, rows, d.nz, W, bits);
+  run_init<<<threads, 128, 0, s>>>(q, words, par);
+  run_link<<<threads, 128, 0, s>>>(q, words, par);
+  run_flatten<<<threads, 128, 0, s>>>(q, words, par);
+  run_faces<<<(unsigned)std::min<int64_t>((2 * (int64_t)d.ny * W + 127) / 128, 1216), 128, 0, s>>>(q, par, touch);
+  const unsigned few = std::min(warps, 4864u);
+  if (labels_dev) run_labels<true><<<few, 256, 0, s>>>(q, words, par, touch, transport_dev, cnt);
+  else run_labels<false><<<few, 256, 0, s>>>(q, words, par, touch, transport_dev, cnt);
   OM_CUDA(cudaGetLastError());
   unsigned long long h[2];
-  OM_CUDA(cudaMemcpyAsync(h, cnt.p, sizeof h, cudaMemcpyDeviceToHost, s));
+  OM_CUDA(cudaMemcpyAsync(h, cnt, sizeof h, cudaMemcpyDeviceToHost, s));
   OM_CUDA(cudaStreamSynchronize(s));
   if (npore) *npore = (int64_t)h[0];
   if (ntrans) *ntrans = (int64_t)h[1];
@@ -193,14 +359,8 @@ extern "C" om_status om_label_connectivity_dev(const uint8_t* mask_dev, om_domai
   if (!mask_dev) return fail(OM_EINVAL, "om_label_connectivity_dev: null mask");
   OM_TRY(check_domain(d));
   cudaStream_t s = as_stream(stream);
-  DevBuf<int> lab;
-  int* lp = labels_dev;
-  if (!lp) {
-    OM_TRY(lab.alloc(voxels(d)));
-    lp = lab.p;
-  }
   int64_t np = 0, nt = 0;
-  OM_TRY(label_impl(mask_dev, d, lp, transport_dev, &np, &nt, s));
+  OM_TRY(label_impl(mask_dev, d, labels_dev, transport_dev, &np, &nt, s));
   if (connectivity_out) *connectivity_out = np > 0 ? (double)nt / (double)np : 0.0;
   return OM_OK;
 }

@@ -11,23 +11,25 @@
 // above its last (periodic in z), so that z - 1, z, z + 1 of any column come
 // from one 16-byte word without branches.  16 bytes per 32 voxels (the whole
 // map sits in L2) instead of an 18-entry neighbour table per node.
+#include <algorithm>
+
 #include "lattice.cuh"
 
 namespace om {
 
-__global__ void ns_bits(const uint8_t* nodes, int ny, int nz, int W, int64_t ncol, uint32_t* bits,
-                        uint32_t* cnt) {
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // word index
-  if (k >= ncol * W) return;
-  int64_t c = k / W;
-  int w = (int)(k - c * W);
-  const uint8_t* p = nodes + c * nz;
-  uint32_t b = 0;
-  int z0 = w * 32;
-  int z1 = min(nz, z0 + 32);
-  for (int z = z0; z < z1; ++z) b |= (p[z] ? 1u : 0u) << (z - z0);
-  bits[k] = b;
-  cnt[k] = __popc(b);
+// one warp per word: 32 voxels of a column
+__global__ void ns_bits(const uint8_t* nodes, int nz, int W, int64_t words, uint32_t* bits, uint32_t* cnt) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < words;
+       k += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t c = k / W;
+    const int z = 32 * (int)(k - c * W) + lane;
+    const uint32_t b = __ballot_sync(0xffffffffu, z < nz && nodes[c * nz + z] != 0);
+    if (lane == 0) {
+      bits[k] = b;
+      cnt[k] = __popc(b);
+    }
+  }
 }
 
 // node number of voxel z of the column whose first word is k0, or kNoNode
@@ -37,24 +39,26 @@ __device__ __forceinline__ uint32_t ns_node(const uint32_t* bits, const uint32_t
   return (bits[k] & bit) ? rank[k] + __popc(bits[k] & (bit - 1u)) : kNoNode;
 }
 
+// one warp per word, a lane per voxel: consecutive nodes are written together
 __global__ void ns_fill(const uint32_t* bits, const uint32_t* rank, int ny, int nz, int W,
                         int64_t nwords, uint4* col, uint32_t* coord, int64_t* vox) {
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nwords) return;
-  uint32_t b = bits[k], r = rank[k];
-  int64_t c = k / W;
-  int w = (int)(k - c * W);
-  const int zprev = w == 0 ? nz - 1 : 32 * w - 1;      // below the word's first voxel
-  const int znext = 32 * w + 32 >= nz ? 0 : 32 * w + 32;  // above its last (nz - 1 in the last word)
-  col[k] = make_uint4(b, r, ns_node(bits, rank, c * W, zprev), ns_node(bits, rank, c * W, znext));
-  int x = (int)(c / ny), y = (int)(c - (int64_t)x * ny);
-  while (b) {
-    int bit = __ffs(b) - 1;
-    b &= b - 1;
-    int z = w * 32 + bit;
-    coord[r] = pack_xyz(x, y, z);
-    vox[r] = c * nz + z;
-    ++r;
+  const int lane = threadIdx.x & 31;
+  for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nwords;
+       k += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const uint32_t b = bits[k], r0 = rank[k];
+    const int64_t c = k / W;
+    const int w = (int)(k - c * W);
+    if (lane == 0) {
+      const int zprev = w == 0 ? nz - 1 : 32 * w - 1;         // below the word's first voxel
+      const int znext = 32 * w + 32 >= nz ? 0 : 32 * w + 32;  // above its last (nz - 1 in the last word)
+      col[k] = make_uint4(b, r0, ns_node(bits, rank, c * W, zprev), ns_node(bits, rank, c * W, znext));
+    }
+    if ((b >> lane) & 1u) {
+      const int x = (int)(c / ny), y = (int)(c - (int64_t)x * ny), z = 32 * w + lane;
+      const uint32_t r = r0 + __popc(b & ((1u << lane) - 1u));
+      coord[r] = pack_xyz(x, y, z);
+      vox[r] = c * nz + z;
+    }
   }
 }
 
@@ -147,39 +151,6 @@ __global__ void ns_slow_list(const uint32_t* flag, const uint32_t* pos, int64_t 
 
 using namespace om;
 
-namespace {
-// The neighbour records and the list of slow nodes (see lattice.cuh).
-om_status build_records(om_nodeset* ns, cudaStream_t s) {
-  const om_domain& d = ns->dom;
-  const int64_t nf = ns->nf;
-  const int fit = d.nz <= kRecMaxNz && (int64_t)d.ny * d.nz <= kRecMaxPlane;
-  DevBuf<uint2> r7, r19;
-  DevBuf<uint32_t> flag, pos, list;
-  DevBuf<uint64_t> total;
-  OM_TRY(r7.alloc(nf));
-  OM_TRY(r19.alloc(nf));
-  OM_TRY(flag.alloc(nf));
-  OM_TRY(pos.alloc(nf));
-  OM_TRY(total.alloc(1));
-  const unsigned nb = (unsigned)((nf + 255) / 256);
-  ns_records<<<nb, 256, 0, s>>>(ns->col, ns->coord, nf, d.nx, d.ny, d.nz, ns->W, fit, r7.p, r19.p, flag.p);
-  OM_CUDA(cudaGetLastError());
-  OM_TRY(exclusive_scan_u32(flag.p, pos.p, nf, total.p, s));
-  uint64_t nslow = 0;
-  OM_CUDA(cudaMemcpyAsync(&nslow, total.p, sizeof nslow, cudaMemcpyDeviceToHost, s));
-  OM_CUDA(cudaStreamSynchronize(s));
-  OM_TRY(list.alloc(nslow));
-  ns_slow_list<<<nb, 256, 0, s>>>(flag.p, pos.p, nf, list.p);
-  OM_CUDA(cudaGetLastError());
-  OM_CUDA(cudaStreamSynchronize(s));
-  ns->rec7 = fit ? r7.take() : nullptr;
-  ns->rec19 = fit ? r19.take() : nullptr;
-  ns->slow = list.take();
-  ns->n_slow = (int64_t)nslow;
-  return OM_OK;
-}
-}  // namespace
-
 extern "C" om_status om_nodeset_create(const uint8_t* nodes_dev, om_domain d, void* stream,
                                        om_nodeset** out) {
   if (!nodes_dev || !out) return fail(OM_EINVAL, "om_nodeset_create: null pointer");
@@ -188,59 +159,90 @@ extern "C" om_status om_nodeset_create(const uint8_t* nodes_dev, om_domain d, vo
   const int W = (d.nz + 31) / 32;
   const int64_t ncol = (int64_t)d.nx * d.ny;
   const int64_t nw = ncol * W;
-  DevBuf<uint32_t> bits, cnt, rank;
-  DevBuf<uint64_t> total;
-  DevBuf<unsigned long long> wrap;
-  OM_TRY(bits.alloc(nw));
-  OM_TRY(cnt.alloc(nw));
-  OM_TRY(rank.alloc(nw));
-  OM_TRY(total.alloc(1));
-  OM_TRY(wrap.alloc(1));
-  OM_CUDA(cudaMemsetAsync(wrap.p, 0, sizeof(unsigned long long), s));
-  ns_bits<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(nodes_dev, d.ny, d.nz, W, ncol, bits.p, cnt.p);
-  ns_wrap_links<<<152, 256, 0, s>>>(nodes_dev, d.nx, d.ny, d.nz, wrap.p);
+  // scratch of the column pass
+  StreamBuf tmp(s);
+  size_t at = 0;
+  OM_TRY(tmp.alloc(3 * ((size_t)nw * 4 + 256) + 512));
+  uint64_t* total = carve<uint64_t>(tmp.p, &at, 2);  // nodes, and links across x
+  uint32_t* bits = carve<uint32_t>(tmp.p, &at, nw);
+  uint32_t* cnt = carve<uint32_t>(tmp.p, &at, nw);
+  uint32_t* rank = carve<uint32_t>(tmp.p, &at, nw);
+  OM_CUDA(cudaMemsetAsync(total, 0, 2 * sizeof(uint64_t), s));
+  const unsigned warps = (unsigned)std::min<int64_t>((nw + 7) / 8, 16 * 1216);
+  ns_bits<<<warps, 256, 0, s>>>(nodes_dev, d.nz, W, nw, bits, cnt);
+  ns_wrap_links<<<152, 256, 0, s>>>(nodes_dev, d.nx, d.ny, d.nz, (unsigned long long*)(total + 1));
   OM_CUDA(cudaGetLastError());
-  OM_TRY(exclusive_scan_u32(cnt.p, rank.p, nw, total.p, s));
-  uint64_t nf = 0;
-  unsigned long long nwrap = 0;
-  OM_CUDA(cudaMemcpyAsync(&nf, total.p, sizeof nf, cudaMemcpyDeviceToHost, s));
-  OM_CUDA(cudaMemcpyAsync(&nwrap, wrap.p, sizeof nwrap, cudaMemcpyDeviceToHost, s));
+  OM_TRY(exclusive_scan_u32(cnt, rank, nw, total, s));
+  uint64_t got[2] = {0, 0};
+  OM_CUDA(cudaMemcpyAsync(got, total, sizeof got, cudaMemcpyDeviceToHost, s));
   OM_CUDA(cudaStreamSynchronize(s));
+  const int64_t nf = (int64_t)got[0];
 
   om_nodeset* ns = new om_nodeset();
   ns->dom = d;
   ns->W = W;
   ns->N = voxels(d);
-  ns->nf = (int64_t)nf;
-  ns->pitch = ((int64_t)nf + 63) / 64 * 64;
-  ns->wrap_links = (int64_t)nwrap;
-  DevBuf<uint4> col;
-  DevBuf<uint32_t> coord;
-  DevBuf<int64_t> vox;
-  om_status st = col.alloc(nw);
-  if (st == OM_OK) st = coord.alloc(nf);
-  if (st == OM_OK) st = vox.alloc(nf);
+  ns->nf = nf;
+  ns->pitch = (nf + 63) / 64 * 64;
+  ns->wrap_links = (int64_t)got[1];
+  // one allocation for everything the node set keeps; the slow nodes (lattice.cuh) lie on the
+  // faces of the box, or are all nodes of a box beyond the record fields
+  const int fit = d.nz <= kRecMaxNz && (int64_t)d.ny * d.nz <= kRecMaxPlane;
+  const int64_t inner = std::max(0, d.nx - 2) * (int64_t)std::max(0, d.ny - 2) * std::max(0, d.nz - 2);
+  const int64_t slow_cap = fit ? std::min(nf, ns->N - inner) : nf;
+  DevBuf<uint8_t> mem;
+  const int64_t nrec = fit ? nf : 0;
+  om_status st = mem.alloc((size_t)nw * 16 + (size_t)nf * 12 + (size_t)nrec * 16 + (size_t)slow_cap * 4 + 6 * 256);
+  StreamBuf flags(s);
+  if (st == OM_OK && nf > 0) st = flags.alloc(2 * ((size_t)nf * 4 + 256) + 256 + (fit ? 0 : (size_t)nf * 16 + 512));
   if (st != OM_OK) {
     delete ns;
     return st;
   }
-  ns_fill<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(bits.p, rank.p, d.ny, d.nz, W, nw, col.p,
-                                                      coord.p, vox.p);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
-    delete ns;
-    return cuda_fail(e, "om_nodeset_create fill", __FILE__, __LINE__);
+  at = 0;
+  ns->mem = mem.take();
+  ns->col = carve<uint4>(ns->mem, &at, nw);
+  ns->vox = carve<int64_t>(ns->mem, &at, nf);
+  uint2 *r7 = nullptr, *r19 = nullptr;
+  if (fit) {
+    r7 = carve<uint2>(ns->mem, &at, nf);
+    r19 = carve<uint2>(ns->mem, &at, nf);
   }
-  ns->col = col.take();
-  ns->coord = coord.take();
-  ns->vox = vox.take();
-  if (nf > 0) {
-    om_status rs = build_records(ns, s);
-    if (rs != OM_OK) {
-      om_nodeset_destroy(ns);
-      return rs;
+  ns->coord = carve<uint32_t>(ns->mem, &at, nf);
+  ns->slow = carve<uint32_t>(ns->mem, &at, slow_cap);
+  auto build = [&]() -> om_status {
+    ns_fill<<<warps, 256, 0, s>>>(bits, rank, d.ny, d.nz, W, nw, ns->col, ns->coord, ns->vox);
+    OM_CUDA(cudaGetLastError());
+    uint64_t nslow = 0;
+    if (nf > 0) {
+      size_t f = 0;
+      uint64_t* tslow = carve<uint64_t>(flags.p, &f, 1);
+      uint32_t* flag = carve<uint32_t>(flags.p, &f, nf);
+      uint32_t* pos = carve<uint32_t>(flags.p, &f, nf);
+      if (!fit) {  // written, not kept
+        r7 = carve<uint2>(flags.p, &f, nf);
+        r19 = carve<uint2>(flags.p, &f, nf);
+      }
+      const unsigned nb = (unsigned)((nf + 255) / 256);
+      ns_records<<<nb, 256, 0, s>>>(ns->col, ns->coord, nf, d.nx, d.ny, d.nz, W, fit, r7, r19, flag);
+      OM_CUDA(cudaGetLastError());
+      OM_TRY(exclusive_scan_u32(flag, pos, nf, tslow, s));
+      ns_slow_list<<<nb, 256, 0, s>>>(flag, pos, nf, ns->slow);
+      OM_CUDA(cudaGetLastError());
+      OM_CUDA(cudaMemcpyAsync(&nslow, tslow, sizeof nslow, cudaMemcpyDeviceToHost, s));
     }
+    OM_CUDA(cudaStreamSynchronize(s));
+    ns->n_slow = (int64_t)nslow;
+    if (fit && nf > 0) {
+      ns->rec7 = r7;
+      ns->rec19 = r19;
+    }
+    return OM_OK;
+  };
+  st = build();
+  if (st != OM_OK) {
+    om_nodeset_destroy(ns);
+    return st;
   }
   *out = ns;
   return OM_OK;
@@ -262,12 +264,7 @@ extern "C" om_status om_nodeset_voxels(const om_nodeset* ns, int64_t* voxel_dev,
 
 extern "C" om_status om_nodeset_destroy(om_nodeset* ns) {
   if (!ns) return OM_OK;
-  cudaFree(ns->col);
-  cudaFree(ns->coord);
-  cudaFree(ns->vox);
-  cudaFree(ns->rec7);
-  cudaFree(ns->rec19);
-  cudaFree(ns->slow);
+  cudaFree(ns->mem);
   delete ns;
   return OM_OK;
 }

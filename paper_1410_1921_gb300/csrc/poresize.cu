@@ -484,24 +484,6 @@ __global__ void __launch_bounds__(32 * kMisWarps) mis_gather(const uint8_t* __re
   }
 }
 
-// Stream-ordered scratch, freed on its stream: no device-wide wait, and
-// allowed under stream capture (as the entry point without scratch was).
-struct StreamBuf {
-  void* p = nullptr;
-  cudaStream_t s;
-  explicit StreamBuf(cudaStream_t st) : s(st) {}
-  StreamBuf(const StreamBuf&) = delete;
-  ~StreamBuf() {
-    if (p) cudaFreeAsync(p, s);
-  }
-  bool alloc(size_t bytes) {
-    if (cudaMallocAsync(&p, bytes, s) == cudaSuccess) return true;
-    (void)cudaGetLastError();
-    p = nullptr;
-    return false;
-  }
-};
-
 om_status chord13(const uint8_t* m, const om_domain& d, float* d_nm, int32_t* witness, cudaStream_t s) {
   const double sq2 = std::sqrt(2.0), sq3 = std::sqrt(3.0);
   ChordLines c{};
@@ -521,7 +503,7 @@ om_status chord13(const uint8_t* m, const om_domain& d, float* d_nm, int32_t* wi
     words += k == 2 ? wz : (k == 1 || k == 7 || k == 8 ? wy : wx);
   }
   StreamBuf buf(s);
-  if (!buf.alloc(words * sizeof(uint32_t))) {
+  if (!buf.try_alloc(words * sizeof(uint32_t))) {  // (allowed under stream capture, as the form without scratch)
     chord13_walk<<<4 * 1216, 128, 0, s>>>(m, d.nx, d.ny, d.nz, d.dx_nm, sq2, sq3, d_nm, witness);
     OM_CUDA(cudaGetLastError());
     return OM_OK;
@@ -548,8 +530,7 @@ om_status pore_impl(const uint8_t* m, const om_domain& d, int mode, float* d_nm,
   const int nbx = (d.nx + kBrick - 1) / kBrick, nby = (d.ny + kBrick - 1) / kBrick, nbz = (d.nz + kBrick - 1) / kBrick;
   const int64_t nb = (int64_t)nbx * nby * nbz;
   StreamBuf buf(s);
-  if (!buf.alloc(sizeof(int) * (2 + (size_t)(witness ? 2 : 3) * N + nb)))
-    return fail(OM_ENOMEM, "local_pore_diameter (MIS): scratch allocation failed");
+  OM_TRY(buf.alloc(sizeof(int) * (2 + (size_t)(witness ? 2 : 3) * N + nb)));
   int* info = (int*)buf.p;  // largest r2, and whether there is a solid voxel
   int *g = info + 2, *h = g + N, *top = h + N, *r2 = witness ? witness : top + nb;
   OM_CUDA(cudaMemsetAsync(info, 0, 2 * sizeof(int), s));

@@ -336,9 +336,10 @@ om_status reconstruct_impl(uint64_t seed, const om_domain& d, const om_recon_par
   pl.p = p;
   pl.init(seed);
 
-  DevBuf<int> owner;
-  OM_TRY(owner.alloc(N));
-  fill_int<<<1216, 256, 0, s>>>(owner.p, N, 0x7fffffff);
+  StreamBuf own(s);
+  OM_TRY(own.alloc(sizeof(int) * (size_t)N));
+  int* owner = (int*)own.p;
+  fill_int<<<1216, 256, 0, s>>>(owner, N, 0x7fffffff);
   OM_CUDA(cudaGetLastError());
 
   const double rmean = 0.5 * p.mean_d_nm / d.dx_nm;
@@ -348,8 +349,6 @@ om_status reconstruct_impl(uint64_t seed, const om_domain& d, const om_recon_par
   bool infeasible = false;
   std::vector<DevBall> host_balls;
   std::vector<unsigned long long> cnt;
-  DevBuf<DevBall> dballs;
-  DevBuf<unsigned long long> dcnt;
   while (kstop < 0 && !infeasible) {
     const double need = p.porosity * (double)N - (double)covered;
     int64_t chunk = (int64_t)std::ceil(1.5 * std::max(0.0, need) / vmean) + 16;
@@ -364,20 +363,23 @@ om_status reconstruct_impl(uint64_t seed, const om_domain& d, const om_recon_par
     if (k1 == k0) break;
     host_balls.resize(k1 - k0);
     for (int k = k0; k < k1; ++k) host_balls[k - k0] = to_dev(pl.balls[k], d);
-    OM_TRY(dballs.alloc(k1 - k0));
-    OM_TRY(dcnt.alloc(k1 - k0));
-    OM_CUDA(cudaMemcpyAsync(dballs.p, host_balls.data(), sizeof(DevBall) * (k1 - k0), cudaMemcpyHostToDevice, s));
-    OM_CUDA(cudaMemsetAsync(dcnt.p, 0, sizeof(unsigned long long) * (k1 - k0), s));
+    StreamBuf batch(s);
+    size_t at = 0;
+    OM_TRY(batch.alloc((size_t)(k1 - k0) * (sizeof(DevBall) + sizeof(unsigned long long)) + 512));
+    DevBall* dballs = carve<DevBall>(batch.p, &at, k1 - k0);
+    unsigned long long* dcnt = carve<unsigned long long>(batch.p, &at, k1 - k0);
+    OM_CUDA(cudaMemcpyAsync(dballs, host_balls.data(), sizeof(DevBall) * (k1 - k0), cudaMemcpyHostToDevice, s));
+    OM_CUDA(cudaMemsetAsync(dcnt, 0, sizeof(unsigned long long) * (k1 - k0), s));
     // about 16 blocks for each of the 1216 that are resident, so that large balls do not trail
     const int nb = k1 - k0, split = std::max(1, std::min(64, 16 * 1216 / nb));
-    raster_balls<<<dim3((unsigned)nb, (unsigned)split), 256, 0, s>>>(dballs.p, k0, d.nx, d.ny, d.nz, owner.p);
+    raster_balls<<<dim3((unsigned)nb, (unsigned)split), 256, 0, s>>>(dballs, k0, d.nx, d.ny, d.nz, owner);
     const size_t smem = nb <= kCountSlots ? sizeof(unsigned int) * (size_t)nb : 0;
     OM_CUDA(cudaFuncSetAttribute(count_first_cover, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(unsigned int) * kCountSlots));
-    count_first_cover<<<304, 512, smem, s>>>(owner.p, N, k0, k1, dcnt.p);
+    count_first_cover<<<304, 512, smem, s>>>(owner, N, k0, k1, dcnt);
     OM_CUDA(cudaGetLastError());
     cnt.resize(k1 - k0);
-    OM_CUDA(cudaMemcpyAsync(cnt.data(), dcnt.p, sizeof(unsigned long long) * (k1 - k0), cudaMemcpyDeviceToHost, s));
+    OM_CUDA(cudaMemcpyAsync(cnt.data(), dcnt, sizeof(unsigned long long) * (k1 - k0), cudaMemcpyDeviceToHost, s));
     OM_CUDA(cudaStreamSynchronize(s));
     for (int k = k0; k < k1; ++k) {
       covered += (int64_t)cnt[k - k0];
@@ -388,7 +390,7 @@ om_status reconstruct_impl(uint64_t seed, const om_domain& d, const om_recon_par
     }
   }
   const int klast = kstop >= 0 ? kstop : (int)pl.balls.size() - 1;
-  owner_to_mask<<<1216, 256, 0, s>>>(owner.p, N, klast, mask_dev);
+  owner_to_mask<<<1216, 256, 0, s>>>(owner, N, klast, mask_dev);
   OM_CUDA(cudaGetLastError());
   OM_CUDA(cudaStreamSynchronize(s));
   if (eps_out) *eps_out = (double)covered / (double)N;

@@ -56,13 +56,11 @@ struct Scope {
 om_status transport_nodes(const uint8_t* mask, const om_domain& d, DevBuf<uint8_t>& tr, int64_t& np,
                           int64_t& nt, cudaStream_t s) {
   const int64_t N = voxels(d);
-  DevBuf<uint8_t> m;
-  DevBuf<int> lab;
+  StreamBuf m(s);
   OM_TRY(m.alloc(N));
-  OM_TRY(lab.alloc(N));
   OM_TRY(tr.alloc(N));
   OM_CUDA(cudaMemcpyAsync(m.p, mask, N, cudaMemcpyHostToDevice, s));
-  OM_TRY(label_impl(m.p, d, lab.p, tr.p, &np, &nt, s));
+  OM_TRY(label_impl((const uint8_t*)m.p, d, nullptr, tr.p, &np, &nt, s));
   if (nt == 0) return fail(OM_ENOPERC, "no pore component spans x = 0 .. nx-1");
   return OM_OK;
 }

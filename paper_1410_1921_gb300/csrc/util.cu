@@ -117,15 +117,16 @@ om_status exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint6
     OM_CUDA(cudaGetLastError());
     return OM_OK;
   }
-  DevBuf<uint32_t> sums, offs;
-  OM_TRY(sums.alloc(tiles));
-  OM_TRY(offs.alloc(tiles));
-  scan_tile_sums<<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, sums.p);
+  StreamBuf buf(s);
+  size_t at = 0;
+  OM_TRY(buf.alloc(2 * ((size_t)tiles * sizeof(uint32_t) + 256)));
+  uint32_t* sums = carve<uint32_t>(buf.p, &at, tiles);
+  uint32_t* offs = carve<uint32_t>(buf.p, &at, tiles);
+  scan_tile_sums<<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, sums);
   OM_CUDA(cudaGetLastError());
-  OM_TRY(exclusive_scan_u32(sums.p, offs.p, tiles, nullptr, s));
-  scan_tile_apply<<<(unsigned)tiles, kScanThreads, 0, s>>>(in, out, n, offs.p, total_dev);
+  OM_TRY(exclusive_scan_u32(sums, offs, tiles, nullptr, s));
+  scan_tile_apply<<<(unsigned)tiles, kScanThreads, 0, s>>>(in, out, n, offs, total_dev);
   OM_CUDA(cudaGetLastError());
-  // the buffers are freed by cudaFree, which waits for the stream's work
   return OM_OK;
 }
 
