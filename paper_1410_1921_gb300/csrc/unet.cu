@@ -24,83 +24,83 @@ namespace {
 constexpr int kT = 256;
 inline unsigned blocks(int64_t n, int t = kT) { return (unsigned)std::min<int64_t>((n + t - 1) / t, 1 << 20); }
 
-__global__ void pack_input(const float* x, int cin, int64_t V, bf16* out) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V * 16; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = i / 16;
-    const int c = (int)(i % 16);
-    out[i] = __float2bfloat16_rn(c < cin ? x[v * cin + c] : 0.f);
-  }
-}
-
-// fine grid gf -> coarse grid (gf / 2)
-__global__ void avgpool2(const bf16* in, Grid gf, int C, bf16* out) {
-  const Grid gc{gf.B, gf.D / 2, gf.H / 2, gf.W / 2};
-  const int64_t n = gc.voxels() * C;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    int64_t r = i / C;
-    const int x = (int)(r % gc.W); r /= gc.W;
-    const int y = (int)(r % gc.H); r /= gc.H;
-    const int z = (int)(r % gc.D);
-    const int b = (int)(r / gc.D);
-    float s = 0.f;
-    for (int q = 0; q < 8; ++q) {
-      const int64_t vf = (((int64_t)b * gf.D + 2 * z + (q >> 2)) * gf.H + 2 * y + ((q >> 1) & 1)) * gf.W + 2 * x + (q & 1);
-      s += __bfloat162float(in[vf * C + c]);
-    }
-    out[i] = __float2bfloat16_rn(0.125f * s);
+// input [V][cin] FP32 -> [V][16] BF16, zero-padded: a thread per voxel, two 16-byte stores
+__global__ void pack_input(const float* x, int cin, uint32_t V, bf16* out) {
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
+    const float* p = x + (int64_t)v * cin;
+    union {
+      uint4 u[2];
+      __nv_bfloat16 h[16];
+    } o;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) o.h[c] = __float2bfloat16_rn(c < cin ? p[c] : 0.f);
+    uint4* q = reinterpret_cast<uint4*>(out + (int64_t)v * 16);
+    q[0] = o.u[0];
+    q[1] = o.u[1];
   }
 }
 
 // The element-wise kernels below move 8 channels (one 16-byte vector of
 // BF16) per thread: every channel count and row offset of the network is a
-// multiple of 16.
+// multiple of 16.  The resampling ones take a row of x per block, so that z,
+// y and the batch are divided out once per row and not per element (element
+// by element, with 64-bit divisions, a prediction of 128 x 120 x 136 spent 373 us
+// in these kernels and the operand conversions, 93 us so).
 union V8 {
   uint4 u;
   __nv_bfloat16 h[8];
 };
 
-__device__ __forceinline__ void fine_xyzb(int64_t v, const Grid& g, int& x, int& y, int& z, int& b) {
-  x = (int)(v % g.W);
-  v /= g.W;
-  y = (int)(v % g.H);
-  v /= g.H;
-  z = (int)(v % g.D);
-  b = (int)(v / g.D);
+// row r of grid g: its z, y and batch
+__device__ __forceinline__ void row_zyb(int64_t r, const Grid& g, int& z, int& y, int& b) {
+  const int64_t p = r / g.H;
+  y = (int)(r - p * g.H);
+  b = (int)(p / g.D);
+  z = (int)(p - (int64_t)b * g.D);
 }
 
-__device__ __forceinline__ int64_t coarse_of(const Grid& gf, int x, int y, int z, int b) {
-  return (((int64_t)b * (gf.D / 2) + z / 2) * (gf.H / 2) + y / 2) * (gf.W / 2) + x / 2;
-}
-
-// d(fine) = d(coarse parent) / 8
-__global__ void avgpool2_bwd(const bf16* dout, Grid gf, int C, bf16* din) {
+// fine grid gf -> coarse grid (gf / 2)
+__global__ void avgpool2(const bf16* in, Grid gf, int C, bf16* out) {
+  const Grid gc{gf.B, gf.D / 2, gf.H / 2, gf.W / 2};
   const int C8 = C / 8;
-  const int64_t n = gf.voxels() * C8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c8 = (int)(i % C8);
-    const int64_t v = i / C8;
-    int x, y, z, b;
-    fine_xyzb(v, gf, x, y, z, b);
-    V8 a, o;
-    a.u = *reinterpret_cast<const uint4*>(dout + coarse_of(gf, x, y, z, b) * C + 8 * c8);
+  const int64_t rows = (int64_t)gc.B * gc.D * gc.H;
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    int z, y, b;
+    row_zyb(r, gc, z, y, b);
+    const int64_t f0 = (((int64_t)b * gf.D + 2 * z) * gf.H + 2 * y) * gf.W;
+    for (int i = threadIdx.x; i < gc.W * C8; i += blockDim.x) {
+      const int x = i / C8, c8 = i - x * C8;
+      float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
-    for (int j = 0; j < 8; ++j) o.h[j] = __float2bfloat16_rn(0.125f * __bfloat162float(a.h[j]));
-    *reinterpret_cast<uint4*>(din + v * C + 8 * c8) = o.u;
+      for (int q = 0; q < 8; ++q) {
+        const int64_t vf = f0 + ((int64_t)(q >> 2) * gf.H + ((q >> 1) & 1)) * gf.W + 2 * x + (q & 1);
+        V8 a;
+        a.u = *reinterpret_cast<const uint4*>(in + vf * C + 8 * c8);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[j] += __bfloat162float(a.h[j]);
+      }
+      V8 o;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) o.h[j] = __float2bfloat16_rn(0.125f * s[j]);
+      *reinterpret_cast<uint4*>(out + (r * gc.W + x) * C + 8 * c8) = o.u;
+    }
   }
 }
 
-// nearest 2x: coarse [V_c x C] -> fine rows of ldo, channels [oo, oo + C)
-__global__ void upsample2(const bf16* in, Grid gf, int C, bf16* out, int ldo, int oo) {
+// nearest 2x: coarse [V_c x C] -> fine rows of C
+__global__ void upsample2(const bf16* in, Grid gf, int C, bf16* out) {
   const int C8 = C / 8;
-  const int64_t n = gf.voxels() * C8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c8 = (int)(i % C8);
-    const int64_t v = i / C8;
-    int x, y, z, b;
-    fine_xyzb(v, gf, x, y, z, b);
-    *reinterpret_cast<uint4*>(out + v * ldo + oo + 8 * c8) =
-        *reinterpret_cast<const uint4*>(in + coarse_of(gf, x, y, z, b) * C + 8 * c8);
+  const int64_t rows = (int64_t)gf.B * gf.D * gf.H;
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    int z, y, b;
+    row_zyb(r, gf, z, y, b);
+    const uint4* src = reinterpret_cast<const uint4*>(
+        in + (((int64_t)b * (gf.D / 2) + z / 2) * (gf.H / 2) + y / 2) * (gf.W / 2) * C);
+    uint4* dst = reinterpret_cast<uint4*>(out + r * gf.W * C);
+    for (int i = threadIdx.x; i < gf.W * C8; i += blockDim.x) {
+      const int x = i / C8, c8 = i - x * C8;
+      dst[i] = src[(x / 2) * C8 + c8];
+    }
   }
 }
 
@@ -108,73 +108,142 @@ __global__ void upsample2(const bf16* in, Grid gf, int C, bf16* out, int ldo, in
 __global__ void upsample2_bwd(const bf16* dfine, int ldi, int oi, Grid gf, int C, bf16* dcoarse) {
   const Grid gc{gf.B, gf.D / 2, gf.H / 2, gf.W / 2};
   const int C8 = C / 8;
-  const int64_t n = gc.voxels() * C8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c8 = (int)(i % C8);
-    const int64_t vcoarse = i / C8;
-    int x, y, z, b;
-    fine_xyzb(vcoarse, gc, x, y, z, b);
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int q = 0; q < 8; ++q) {
-      const int64_t vf = (((int64_t)b * gf.D + 2 * z + (q >> 2)) * gf.H + 2 * y + ((q >> 1) & 1)) * gf.W + 2 * x + (q & 1);
-      V8 a;
-      a.u = *reinterpret_cast<const uint4*>(dfine + vf * ldi + oi + 8 * c8);
+  const int64_t rows = (int64_t)gc.B * gc.D * gc.H;
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    int z, y, b;
+    row_zyb(r, gc, z, y, b);
+    const int64_t f0 = (((int64_t)b * gf.D + 2 * z) * gf.H + 2 * y) * gf.W;
+    for (int i = threadIdx.x; i < gc.W * C8; i += blockDim.x) {
+      const int x = i / C8, c8 = i - x * C8;
+      float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(a.h[j]);
+      for (int q = 0; q < 8; ++q) {
+        const int64_t vf = f0 + ((int64_t)(q >> 2) * gf.H + ((q >> 1) & 1)) * gf.W + 2 * x + (q & 1);
+        V8 a;
+        a.u = *reinterpret_cast<const uint4*>(dfine + vf * ldi + oi + 8 * c8);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(a.h[j]);
+      }
+      V8 o;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) o.h[j] = __float2bfloat16_rn(acc[j]);
+      *reinterpret_cast<uint4*>(dcoarse + (r * gc.W + x) * C + 8 * c8) = o.u;
     }
-    V8 o;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) o.h[j] = __float2bfloat16_rn(acc[j]);
-    *reinterpret_cast<uint4*>(dcoarse + vcoarse * C + 8 * c8) = o.u;
   }
 }
 
-// gradient at the pre-activation: g * [y > 0]; g read from rows of ldg at og
-__global__ void relu_bwd(const bf16* g, int ldg, int og, const bf16* y, int N, int64_t V, bf16* out) {
-  const int N8 = N / 8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V * N8; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = i / N8;
-    const int c8 = (int)(i % N8);
-    V8 yy, gg, o;
-    yy.u = *reinterpret_cast<const uint4*>(y + v * N + 8 * c8);
-    gg.u = *reinterpret_cast<const uint4*>(g + v * ldg + og + 8 * c8);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) o.h[j] = __bfloat162float(yy.h[j]) > 0.f ? gg.h[j] : __float2bfloat16_rn(0.f);
-    *reinterpret_cast<uint4*>(out + v * N + 8 * c8) = o.u;
-  }
-}
+// The gradient at a pre-activation, out = g [y > 0], and the bias gradient
+// db[c] += sum_v out[v][c], in one pass.  g is formed on the way:
+//   kGradRows  read from rows of ldg at og;
+//   kGradSkip  what the pooling below and the decoder's skip send to an
+//              encoder level: BF16(BF16(coarse / 8) + skip), coarse rows of N
+//              of the level below, skip from rows of ldg at og;
+//   kGradHead  the head's: sum_o dy[v][o] w[c][o]; with y the head's input,
+//              the head's own gradients dw[c][o] += y dy, dhb[o] += dy are
+//              summed in the same pass (up to kHeadOut outputs).
+// A thread keeps its 8 channels over every voxel it visits; the block's
+// threads of a channel group are summed in shared memory, then added with
+// one atomic per channel.  As separate passes (ReLU, bias sums, pooling
+// gradient, skip addition, head) these took 510 us of a training step on
+// 4 x 64^3 (channels 32-64-128), 238 us so; bound by their reads and writes.
+enum { kGradRows = 0, kGradSkip = 1, kGradHead = 2 };
+constexpr int kHeadOut = 4;
+struct GradArgs {
+  const bf16* g;
+  int ldg, og;
+  const bf16* coarse;
+  Grid gf;           // the fine grid (kGradSkip)
+  const float *dy, *w;
+  int O;             // head outputs
+  float *dw, *dhb;   // head gradients (null: not summed here)
+  const bf16* y;
+  int N;
+  uint32_t V;
+  bf16* out;
+  float* db;
+};
 
-// a[i] += b (rows of ldb at ob), BF16; 8 channels per thread
-__global__ void add_into(bf16* a, int N, int64_t V, const bf16* b, int ldb, int ob) {
-  const int N8 = N / 8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V * N8; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = i / N8;
-    const int c8 = (int)(i % N8);
-    V8 x, y;
-    x.u = *reinterpret_cast<const uint4*>(a + v * N + 8 * c8);
-    y.u = *reinterpret_cast<const uint4*>(b + v * ldb + ob + 8 * c8);
+template <int SRC>
+__global__ void __launch_bounds__(256) relu_grad(GradArgs a) {
+  extern __shared__ float sh[];  // [8][256]
+  const int N8 = a.N / 8, lanes = 256 / N8, c8 = threadIdx.x % N8, lane = threadIdx.x / N8;
+  const bool live = lane < lanes;
+  constexpr int kSums = SRC == kGradHead ? 1 + kHeadOut : 1;
+  float acc[kSums][8], accb[kHeadOut] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int j = 0; j < 8; ++j) x.h[j] = __float2bfloat16_rn(__bfloat162float(x.h[j]) + __bfloat162float(y.h[j]));
-    *reinterpret_cast<uint4*>(a + v * N + 8 * c8) = x.u;
-  }
-}
-
-// db[c] += sum_v g[v][c]: thread t of a block sums channel t % N over the
-// block's voxels t / N, t / N + lanes, ... (coalesced rows), then the lanes
-// of a channel are reduced in shared memory and added to db
-__global__ void bias_grad(const bf16* g, int N, int64_t V, float* db) {
-  extern __shared__ float sh[];
-  const int lanes = blockDim.x / N, c = threadIdx.x % N, lane = threadIdx.x / N;
-  float acc = 0.f;
-  if (lane < lanes)
-    for (int64_t v = (int64_t)blockIdx.x * lanes + lane; v < V; v += (int64_t)gridDim.x * lanes)
-      acc += __bfloat162float(g[v * N + c]);
-  sh[threadIdx.x] = lane < lanes ? acc : 0.f;
-  __syncthreads();
-  if (threadIdx.x < N) {
-    float t = 0.f;
-    for (int l = 0; l < lanes; ++l) t += sh[l * N + threadIdx.x];
-    atomicAdd(&db[threadIdx.x], t);
+  for (int k = 0; k < kSums; ++k)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[k][j] = 0.f;
+  if (live)
+    for (uint32_t v = blockIdx.x * lanes + lane; v < a.V; v += gridDim.x * lanes) {
+      V8 yy, gg, o;
+      yy.u = *reinterpret_cast<const uint4*>(a.y + (int64_t)v * a.N + 8 * c8);
+      if (SRC == kGradHead) {
+        float d[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        for (int k = 0; k < a.O; ++k) {
+          const float t = a.dy[(int64_t)v * a.O + k];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) d[j] += t * a.w[(8 * c8 + j) * a.O + k];
+        }
+        if (a.dw) {
+#pragma unroll
+          for (int k = 0; k < kHeadOut; ++k)
+            if (k < a.O) {
+              const float t = a.dy[(int64_t)v * a.O + k];
+              accb[k] += t;
+#pragma unroll
+              for (int j = 0; j < 8; ++j) acc[SRC == kGradHead ? 1 + k : 0][j] += __bfloat162float(yy.h[j]) * t;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) gg.h[j] = __float2bfloat16_rn(d[j]);
+      } else {
+        gg.u = *reinterpret_cast<const uint4*>(a.g + (int64_t)v * a.ldg + a.og + 8 * c8);
+        if (SRC == kGradSkip) {
+          const uint32_t W = a.gf.W, H = a.gf.H, D = a.gf.D;
+          const uint32_t r = v / W, x = v - r * W, p = r / H, yv = r - p * H, bb = p / D, z = p - bb * D;
+          const int64_t vc = (((int64_t)bb * (D / 2) + z / 2) * (H / 2) + yv / 2) * (W / 2) + x / 2;
+          V8 cc;
+          cc.u = *reinterpret_cast<const uint4*>(a.coarse + vc * a.N + 8 * c8);
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            gg.h[j] = __float2bfloat16_rn(__bfloat162float(__float2bfloat16_rn(0.125f * __bfloat162float(cc.h[j]))) +
+                                          __bfloat162float(gg.h[j]));
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        o.h[j] = __bfloat162float(yy.h[j]) > 0.f ? gg.h[j] : __float2bfloat16_rn(0.f);
+        acc[0][j] += __bfloat162float(o.h[j]);
+      }
+      *reinterpret_cast<uint4*>(a.out + (int64_t)v * a.N + 8 * c8) = o.u;
+    }
+  auto reduce = [&](const float (&t)[8], auto put) {
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sh[j * 256 + threadIdx.x] = live ? t[j] : 0.f;
+    __syncthreads();
+    for (int c = threadIdx.x; c < a.N; c += 256) {
+      float sum = 0.f;
+      for (int l = 0; l < lanes; ++l) sum += sh[(c & 7) * 256 + l * N8 + (c >> 3)];
+      put(c, sum);
+    }
+  };
+  reduce(acc[0], [&](int c, float t) { atomicAdd(&a.db[c], t); });
+  if (SRC == kGradHead && a.dw) {
+#pragma unroll
+    for (int k = 0; k < kHeadOut; ++k)
+      if (k < a.O) {
+        reduce(acc[SRC == kGradHead ? 1 + k : 0], [&](int c, float t) { atomicAdd(&a.dw[c * a.O + k], t); });
+        __syncthreads();
+        sh[threadIdx.x] = live && c8 == 0 ? accb[k] : 0.f;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          float t = 0.f;
+          for (int l = 0; l < lanes; ++l) t += sh[l * N8];
+          atomicAdd(&a.dhb[k], t);
+        }
+      }
   }
 }
 
@@ -222,24 +291,7 @@ __global__ void mse_grad(const float* y, const float* t, const uint8_t* m, int O
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc);
 }
 
-// head backward: dw[c][o] += sum_v x[v][c] dy[v][o]; db[o] += sum_v dy; dx[v][c] = sum_o dy w[c][o]
-__global__ void head_bwd_dx(const float* dy, const float* w, int C, int O, int64_t V, bf16* dx) {
-  const int C8 = C / 8;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V * C8; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = i / C8;
-    const int c0 = (int)(i % C8) * 8;
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int o = 0; o < O; ++o) {
-      const float d = dy[v * O + o];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] += d * w[(c0 + j) * O + o];
-    }
-    V8 q;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) q.h[j] = __float2bfloat16_rn(acc[j]);
-    *reinterpret_cast<uint4*>(dx + v * C + c0) = q.u;
-  }
-}
+// The head's gradients where it has more than kHeadOut outputs:
 // dw[c][o] and db[o] for o in [o0, o0 + 4): thread t of a block takes channel t % C of the
 // voxels t / C, t / C + lanes, ... (coalesced rows); the lanes are reduced in shared memory
 __global__ void head_bwd_dw(const bf16* x, const float* dy, int C, int O, int o0, int64_t V, float* dw, float* db) {
@@ -277,24 +329,31 @@ __global__ void head_bwd_dw(const bf16* x, const float* dy, int C, int O, int o0
   }
 }
 
-// FP32 master W[27][K][N] -> forward operand WT[27][N][K] (BF16)
-__global__ void weights_fwd(const float* W, int K, int N, bf16* WT) {
-  const int64_t n = 27LL * K * N;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int k = (int)(i / ((int64_t)K * N));
-    const int r = (int)(i % ((int64_t)K * N));
-    const int ci = r / N, co = r % N;
-    WT[((int64_t)k * N + co) * K + ci] = __float2bfloat16_rn(W[i]);
-  }
-}
-// data-gradient operand WD[27][K][N] = W[26 - k][K][N] (BF16): the forward
-// kernel with inputs dY (N channels) and output channels K
-__global__ void weights_dgrad(const float* W, int K, int N, bf16* WD) {
-  const int64_t n = 27LL * K * N;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int k = (int)(i / ((int64_t)K * N));
-    const int64_t r = i % ((int64_t)K * N);
-    WD[i] = __float2bfloat16_rn(W[(int64_t)(26 - k) * K * N + r]);
+// Every convolution's operands from the FP32 master weights in one launch
+// (a launch per convolution and operand was 20 to 28 of them): FWD the
+// forward operand WT[27][N][K] of W[27][K][N], else the data gradient's
+// WD[27][K][N] = W[26 - k][K][N], the forward kernel with inputs dY (N
+// channels) and output channels K.  blockIdx.y = convolution.
+constexpr int kMaxConvs = 24;
+struct OperandTable {
+  const float* W[kMaxConvs];
+  bf16* out[kMaxConvs];
+  int K[kMaxConvs], N[kMaxConvs];
+};
+template <bool FWD>
+__global__ void convert_weights(const __grid_constant__ OperandTable t) {
+  const int K = t.K[blockIdx.y], N = t.N[blockIdx.y];
+  const uint32_t per = (uint32_t)K * N, n = 27u * per;
+  const float* W = t.W[blockIdx.y];
+  bf16* out = t.out[blockIdx.y];
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t k = i / per, r = i - k * per;
+    if (FWD) {
+      const uint32_t ci = r / N, co = r - ci * N;
+      out[((uint64_t)k * N + co) * K + ci] = __float2bfloat16_rn(W[i]);
+    } else {
+      out[i] = __float2bfloat16_rn(W[(26u - k) * per + r]);
+    }
   }
 }
 
@@ -363,6 +422,8 @@ struct om_unet {
   // gradients (scratch)
   std::vector<Buf<bf16>> d1, d2, dcat, ds;
   Buf<double> loss;
+  // the BF16 operands are those of the present weights (cleared where the weights change)
+  bool wt_ready = false, wd_ready = false;
   Buf<int> tc_err;  // set by a tensor-core convolution whose wait ran out
 };
 
@@ -572,17 +633,13 @@ om_status wgrad_tc(om_unet* U, const Conv& c, const bf16* x1, int ld1, int o1, c
   return OM_OK;
 }
 
-// dW += the weight gradient of conv c, db += its bias gradient, for the pre-activation gradient dyp
+// dW += the weight gradient of conv c for the pre-activation gradient dyp (its bias gradient: relu_grad)
 om_status conv_wgrad(om_unet* U, const Conv& c, const bf16* x1, int ld1, int o1, const bf16* x2, int ld2, int o2,
                      const bf16* dyp, const Grid& g, cudaStream_t s) {
   if (c.cout % 16 || c.cout > 256 || c.cin1 % 8 || c.cin2 % 8 || ld1 % 8 || o1 % 8 ||
       (c.cin2 > 0 && (ld2 % 8 || o2 % 8)))
     return fail(OM_EINVAL, "U-Net: weight-gradient shape outside the tensor-core kernel's layout");
-  OM_TRY(wgrad_tc(U, c, x1, ld1, o1, x2, ld2, o2, dyp, g, s));
-  bias_grad<<<std::min<int64_t>(blocks(g.voxels() * c.cout), 1216), kT, kT * sizeof(float), s>>>(
-      dyp, c.cout, g.voxels(), U->g + c.b_off);
-  OM_CUDA(cudaGetLastError());
-  return OM_OK;
+  return wgrad_tc(U, c, x1, ld1, o1, x2, ld2, o2, dyp, g, s);
 }
 
 Grid level_grid(const Grid& g, int l) { return Grid{g.B, g.D >> l, g.H >> l, g.W >> l}; }
@@ -616,11 +673,19 @@ om_status prepare(om_unet* U, const Grid& g) {
   return OM_OK;
 }
 
-om_status refresh_operands(om_unet* U, cudaStream_t s) {
+// the forward (or data-gradient) operands of the present weights
+om_status refresh_operands(om_unet* U, bool fwd, cudaStream_t s) {
+  bool& ready = fwd ? U->wt_ready : U->wd_ready;
+  if (ready) return OM_OK;
+  OperandTable t{};
+  int n = 0, most = 0;
   auto conv = [&](Conv& c) {
-    const int K = c.cin1 + c.cin2;
-    weights_fwd<<<blocks(27LL * K * c.cout), kT, 0, s>>>(U->w + c.w_off, K, c.cout, c.wt);
-    weights_dgrad<<<blocks(27LL * K * c.cout), kT, 0, s>>>(U->w + c.w_off, K, c.cout, c.wd);
+    t.W[n] = U->w + c.w_off;
+    t.out[n] = fwd ? c.wt : c.wd;
+    t.K[n] = c.cin1 + c.cin2;
+    t.N[n] = c.cout;
+    most = std::max(most, 27 * t.K[n] * t.N[n]);
+    ++n;
   };
   for (int l = 0; l < U->L; ++l) {
     conv(U->enc1[l]);
@@ -630,20 +695,37 @@ om_status refresh_operands(om_unet* U, cudaStream_t s) {
       conv(U->dec2[l]);
     }
   }
+  const dim3 grid(std::min<unsigned>(blocks(most), 608), (unsigned)n);
+  if (fwd) convert_weights<true><<<grid, kT, 0, s>>>(t);
+  else convert_weights<false><<<grid, kT, 0, s>>>(t);
+  OM_CUDA(cudaGetLastError());
+  ready = true;
+  return OM_OK;
+}
+
+unsigned row_blocks(const Grid& g) { return (unsigned)std::min<int64_t>((int64_t)g.B * g.D * g.H, 8 * 1216); }
+
+om_status launch_relu_grad(int src, const GradArgs& a, cudaStream_t s) {
+  const int lanes = 256 / (a.N / 8);
+  const unsigned nb = (unsigned)std::min<int64_t>(((int64_t)a.V + lanes - 1) / lanes, 1216);
+  const size_t smem = 8 * 256 * sizeof(float);
+  if (src == kGradRows) relu_grad<kGradRows><<<nb, 256, smem, s>>>(a);
+  else if (src == kGradSkip) relu_grad<kGradSkip><<<nb, 256, smem, s>>>(a);
+  else relu_grad<kGradHead><<<nb, 256, smem, s>>>(a);
   OM_CUDA(cudaGetLastError());
   return OM_OK;
 }
 
 om_status forward(om_unet* U, const float* x, const Grid& g, cudaStream_t s) {
   OM_TRY(prepare(U, g));
-  OM_TRY(refresh_operands(U, s));
+  OM_TRY(refresh_operands(U, true, s));
   const int L = U->L;
-  pack_input<<<blocks(g.voxels() * 16), kT, 0, s>>>(x, U->in_ch, g.voxels(), U->x0.p);
+  pack_input<<<std::min<unsigned>(blocks(g.voxels()), 16 * 1216), kT, 0, s>>>(x, U->in_ch, (uint32_t)g.voxels(), U->x0.p);
   for (int l = 0; l < L; ++l) {
     const Grid gl = level_grid(g, l);
     const bf16* in = l == 0 ? U->x0.p : U->in[l].p;
     const int cin = l == 0 ? 16 : U->ch[l - 1];
-    if (l > 0) avgpool2<<<blocks(gl.voxels() * cin), kT, 0, s>>>(U->s[l - 1].p, level_grid(g, l - 1), cin, U->in[l].p);
+    if (l > 0) avgpool2<<<row_blocks(gl), kT, 0, s>>>(U->s[l - 1].p, level_grid(g, l - 1), cin, U->in[l].p);
     OM_TRY(conv_forward(U, U->enc1[l], in, cin, 0, nullptr, 0, 0, U->a[l].p, gl, s));
     OM_TRY(conv_forward(U, U->enc2[l], U->a[l].p, U->ch[l], 0, nullptr, 0, 0, U->s[l].p, gl, s));
   }
@@ -651,7 +733,7 @@ om_status forward(om_unet* U, const float* x, const Grid& g, cudaStream_t s) {
     const Grid gl = level_grid(g, l);
     const bf16* below = l + 1 == L - 1 ? U->s[L - 1].p : U->h[l + 1].p;
     const int cb = U->ch[l + 1];
-    upsample2<<<blocks(gl.voxels() * cb / 8), kT, 0, s>>>(below, gl, cb, U->u[l].p, cb, 0);
+    upsample2<<<row_blocks(gl), kT, 0, s>>>(below, gl, cb, U->u[l].p);
     OM_TRY(conv_forward(U, U->dec1[l], U->u[l].p, cb, 0, U->s[l].p, U->ch[l], 0, U->b[l].p, gl, s));
     OM_TRY(conv_forward(U, U->dec2[l], U->b[l].p, U->ch[l], 0, nullptr, 0, 0, U->h[l].p, gl, s));
   }
@@ -673,49 +755,68 @@ om_status backward(om_unet* U, const float* t, const uint8_t* mk, const Grid& g,
   mask_count<<<std::min<unsigned>(blocks(V), 1216), kT, 0, s>>>(mk, V, U->loss.p + 1);
   mse_grad<<<std::min<unsigned>(blocks(V * U->out_ch), 1216), kT, 0, s>>>(U->out.p, t, mk, U->out_ch, V, U->loss.p + 1,
                                                                            U->dout.p, U->loss.p);
-  // head
+  OM_TRY(refresh_operands(U, false, s));
   const int c0 = U->ch[0];
   const bf16* top = L > 1 ? U->h[0].p : U->s[0].p;
-  for (int o0 = 0; o0 < U->out_ch; o0 += 4)
-    head_bwd_dw<<<1216, kT, 8 * kT * sizeof(float), s>>>(top, U->dout.p, c0, U->out_ch, o0, V, U->g + U->head_w,
-                                                         U->g + U->head_b);
-  head_bwd_dx<<<blocks(V * c0 / 8), kT, 0, s>>>(U->dout.p, U->w + U->head_w, c0, U->out_ch, V, U->d1[0].p);
+  const bool head_fused = U->out_ch <= kHeadOut;
+  if (!head_fused)
+    for (int o0 = 0; o0 < U->out_ch; o0 += 4)
+      head_bwd_dw<<<1216, kT, 8 * kT * sizeof(float), s>>>(top, U->dout.p, c0, U->out_ch, o0, V, U->g + U->head_w,
+                                                           U->g + U->head_b);
+  // pre-activation gradient of the activation y (N channels) of conv c, and c's bias gradient
+  auto grad_args = [&](const Conv& c, const bf16* y, const Grid& gl, bf16* out) {
+    GradArgs a{};
+    a.y = y, a.N = c.cout, a.V = (uint32_t)gl.voxels(), a.out = out, a.db = U->g + c.b_off;
+    return a;
+  };
+  auto rows_grad = [&](const Conv& c, const bf16* g, const bf16* y, const Grid& gl, bf16* out) {
+    GradArgs a = grad_args(c, y, gl, out);
+    a.g = g, a.ldg = c.cout, a.og = 0;
+    return launch_relu_grad(kGradRows, a, s);
+  };
+  auto head_grad = [&](const Conv& c, bf16* out) {
+    GradArgs a = grad_args(c, top, g, out);
+    a.dy = U->dout.p, a.w = U->w + U->head_w, a.O = U->out_ch;
+    if (head_fused) a.dw = U->g + U->head_w, a.dhb = U->g + U->head_b;
+    return launch_relu_grad(kGradHead, a, s);
+  };
   // decoder, top level down: d1[l] holds the gradient of the level's output h_l
   for (int l = 0; l + 1 < L; ++l) {
     const Grid gl = level_grid(g, l);
-    const int64_t Vl = gl.voxels();
     const int c = U->ch[l], cb = U->ch[l + 1];
     // h_l = relu(conv(b_l))
-    relu_bwd<<<blocks(Vl * c / 8), kT, 0, s>>>(U->d1[l].p, c, 0, U->h[l].p, c, Vl, U->d2[l].p);
+    if (l == 0) OM_TRY(head_grad(U->dec2[l], U->d2[l].p));
+    else OM_TRY(rows_grad(U->dec2[l], U->d1[l].p, U->h[l].p, gl, U->d2[l].p));
     OM_TRY(conv_wgrad(U, U->dec2[l], U->b[l].p, c, 0, nullptr, 0, 0, U->d2[l].p, gl, s));
     OM_TRY(conv_dgrad(U, U->dec2[l], U->d2[l].p, U->d1[l].p, gl, s));
     // b_l = relu(conv(concat(u_l, s_l)))
-    relu_bwd<<<blocks(Vl * c / 8), kT, 0, s>>>(U->d1[l].p, c, 0, U->b[l].p, c, Vl, U->d2[l].p);
+    OM_TRY(rows_grad(U->dec1[l], U->d1[l].p, U->b[l].p, gl, U->d2[l].p));
     OM_TRY(conv_wgrad(U, U->dec1[l], U->u[l].p, cb, 0, U->s[l].p, c, 0, U->d2[l].p, gl, s));
     OM_TRY(conv_dgrad(U, U->dec1[l], U->d2[l].p, U->dcat[l].p, gl, s));
     // u_l = up(h_{l+1}) (or s_{L-1} at the bottom): gradient of the level below
-    upsample2_bwd<<<blocks(level_grid(g, l + 1).voxels() * cb / 8), kT, 0, s>>>(U->dcat[l].p, cb + c, 0, gl, cb,
-                                                                            U->d1[l + 1].p);
+    upsample2_bwd<<<row_blocks(level_grid(g, l + 1)), kT, 0, s>>>(U->dcat[l].p, cb + c, 0, gl, cb, U->d1[l + 1].p);
   }
-  // encoder, bottom level up: ds[l] = gradient of s_l
+  // encoder, bottom level up
   for (int l = L - 1; l >= 0; --l) {
     const Grid gl = level_grid(g, l);
-    const int64_t Vl = gl.voxels();
     const int c = U->ch[l];
     const int cin = l == 0 ? 16 : U->ch[l - 1];
-    // s_l receives: from the level below (pooling) and from the decoder's skip
-    if (l == L - 1) {
-      OM_CUDA(cudaMemcpyAsync(U->ds[l].p, U->d1[l].p, sizeof(bf16) * Vl * c, cudaMemcpyDeviceToDevice, s));
+    // s_l = relu(conv(a_l)) receives: from the level below (pooling) and from the decoder's skip
+    if (L == 1) {
+      OM_TRY(head_grad(U->enc2[l], U->d1[l].p));
+    } else if (l == L - 1) {
+      OM_TRY(rows_grad(U->enc2[l], U->d1[l].p, U->s[l].p, gl, U->ds[l].p));
     } else {
-      avgpool2_bwd<<<blocks(Vl * c / 8), kT, 0, s>>>(U->d2[l + 1].p, gl, c, U->ds[l].p);
-      add_into<<<blocks(Vl * c / 8), kT, 0, s>>>(U->ds[l].p, c, Vl, U->dcat[l].p, U->ch[l + 1] + c, U->ch[l + 1]);
+      GradArgs a = grad_args(U->enc2[l], U->s[l].p, gl, U->ds[l].p);
+      a.g = U->dcat[l].p, a.ldg = U->ch[l + 1] + c, a.og = U->ch[l + 1];
+      a.coarse = U->d2[l + 1].p, a.gf = gl;
+      OM_TRY(launch_relu_grad(kGradSkip, a, s));
     }
-    // s_l = relu(conv(a_l))
-    relu_bwd<<<blocks(Vl * c / 8), kT, 0, s>>>(U->ds[l].p, c, 0, U->s[l].p, c, Vl, U->d1[l].p);
-    OM_TRY(conv_wgrad(U, U->enc2[l], U->a[l].p, c, 0, nullptr, 0, 0, U->d1[l].p, gl, s));
-    OM_TRY(conv_dgrad(U, U->enc2[l], U->d1[l].p, U->d2[l].p, gl, s));
+    const bf16* dp = L == 1 ? U->d1[l].p : U->ds[l].p;
+    OM_TRY(conv_wgrad(U, U->enc2[l], U->a[l].p, c, 0, nullptr, 0, 0, dp, gl, s));
+    OM_TRY(conv_dgrad(U, U->enc2[l], dp, U->d2[l].p, gl, s));
     // a_l = relu(conv(in_l))
-    relu_bwd<<<blocks(Vl * c / 8), kT, 0, s>>>(U->d2[l].p, c, 0, U->a[l].p, c, Vl, U->d1[l].p);
+    OM_TRY(rows_grad(U->enc1[l], U->d2[l].p, U->a[l].p, gl, U->d1[l].p));
     const bf16* in = l == 0 ? U->x0.p : U->in[l].p;
     OM_TRY(conv_wgrad(U, U->enc1[l], in, cin, 0, nullptr, 0, 0, U->d1[l].p, gl, s));
     // d2[l] = gradient of in_l (pooled s_{l-1}); not needed at the input
@@ -864,6 +965,7 @@ extern "C" om_status om_unet_get_params(const om_unet* U, float* dst_dev, void* 
 
 extern "C" om_status om_unet_set_params(om_unet* U, const float* src_dev, void* stream) {
   if (!U || !src_dev) return fail(OM_EINVAL, "om_unet_set_params: null pointer");
+  U->wt_ready = U->wd_ready = false;
   OM_CUDA(cudaMemcpyAsync(U->w, src_dev, sizeof(float) * U->nparam, cudaMemcpyDeviceToDevice, as_stream(stream)));
   return OM_OK;
 }
@@ -880,9 +982,14 @@ extern "C" om_status om_unet_forward(om_unet* U, const float* x, int32_t B, int3
   const Grid g{B, D, H, W};
   OM_TRY(check_grid(U, g));
   cudaStream_t s = as_stream(stream);
-  OM_TRY(forward(U, x, g, s));
-  OM_CUDA(cudaMemcpyAsync(y, U->out.p, sizeof(float) * g.voxels() * U->out_ch, cudaMemcpyDeviceToDevice, s));
-  return check_tc(U, s);
+  auto go = [&]() -> om_status {
+    OM_TRY(forward(U, x, g, s));
+    OM_CUDA(cudaMemcpyAsync(y, U->out.p, sizeof(float) * g.voxels() * U->out_ch, cudaMemcpyDeviceToDevice, s));
+    return check_tc(U, s);
+  };
+  const om_status st = go();
+  if (st != OM_OK) U->wt_ready = U->wd_ready = false;  // whatever was enqueued is not waited for
+  return st;
 }
 
 extern "C" om_status om_unet_backward(om_unet* U, const float* x, const float* t, const uint8_t* m, int32_t B,
@@ -891,8 +998,10 @@ extern "C" om_status om_unet_backward(om_unet* U, const float* x, const float* t
   const Grid g{B, D, H, W};
   OM_TRY(check_grid(U, g));
   cudaStream_t s = as_stream(stream);
-  OM_TRY(forward(U, x, g, s));
-  return backward(U, t, m, g, loss_out, s);
+  om_status st = forward(U, x, g, s);
+  if (st == OM_OK) st = backward(U, t, m, g, loss_out, s);
+  if (st != OM_OK) U->wt_ready = U->wd_ready = false;  // whatever was enqueued is not waited for
+  return st;
 }
 
 namespace om {
@@ -942,6 +1051,7 @@ extern "C" om_status om_unet_train_step(om_unet* U, const float* x, const float*
   ++U->step;
   const float b1 = 0.9f, b2 = 0.999f;
   const float bc1 = 1.f - std::pow(b1, (float)U->step), bc2 = 1.f - std::pow(b2, (float)U->step);
+  U->wt_ready = U->wd_ready = false;
   adam_step<<<blocks(U->nparam), kT, 0, s>>>(U->w, U->g, U->m, U->v, U->nparam, lr, b1, b2, 1e-8f, bc1, bc2);
   OM_CUDA(cudaGetLastError());
   return OM_OK;
