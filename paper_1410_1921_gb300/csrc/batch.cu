@@ -120,12 +120,14 @@ __device__ __forceinline__ void diff_group_tile(const DiffArgs<T>& a, const Grou
 
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(kTile, MINB) flow_batch_sweep(FlowArgs<T> a, const __grid_constant__ GroupDesc g) {
+  grid_trigger();
   const int nw = g.tile0[g.n];
   for (int w = blockIdx.x; w < nw; w += gridDim.x) flow_group_tile<T, ODD>(a, g, w);
 }
 
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(kTile, MINB) diff_batch_sweep(DiffArgs<T> a, const __grid_constant__ GroupDesc g) {
+  grid_trigger();
   const int nw = g.tile0[g.n];
   for (int w = blockIdx.x; w < nw; w += gridDim.x) diff_group_tile<T, ODD>(a, g, w);
 }
@@ -221,6 +223,7 @@ __global__ void barrier_selftest(GridBar* bar, int rounds, unsigned extra, unsig
 // nodes are [off, off + nf) of the arena, one thread per node.
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(kTile, MINB) flow_solo_sweep(FlowArgs<T> a, uint32_t off) {
+  grid_trigger();
   const uint32_t ln = blockIdx.x * blockDim.x + threadIdx.x;
   if (ln >= a.nf) return;
   flow_node<T, ODD>(a, off + ln, ln);
@@ -234,6 +237,7 @@ __global__ void __launch_bounds__(kTile, MINB) flow_solo_sweep(FlowArgs<T> a, ui
 // for a solo item, whose arena offset is a multiple of 32).
 template <class T>
 __global__ void __launch_bounds__(kTile) flow_solo_strided(FlowArgs<T> a, uint32_t off) {
+  grid_trigger();
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t ln = blockIdx.x * blockDim.x + threadIdx.x;
   if (ln >= a.nf) return;
@@ -251,6 +255,7 @@ __global__ void __launch_bounds__(kTile) flow_solo_strided(FlowArgs<T> a, uint32
 
 template <class T>
 __global__ void __launch_bounds__(kTile) flow_solo_pair(FlowArgs<T> a, uint32_t off) {
+  grid_trigger();
   const uint32_t head = off & 1u;
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (head && t == 0) flow_node_at<T, false>(a, off, 0u);
@@ -262,6 +267,7 @@ __global__ void __launch_bounds__(kTile) flow_solo_pair(FlowArgs<T> a, uint32_t 
 
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(kTile, MINB) diff_solo_sweep(DiffArgs<T> a, uint32_t off) {
+  grid_trigger();
   const uint32_t ln = blockIdx.x * blockDim.x + threadIdx.x;
   if (ln >= a.nf) return;
   diff_node<T, ODD>(a, off + ln, ln);
@@ -790,19 +796,19 @@ void launch_flow_t(const om_batch* b, bool odd, int grid, int g, int form, cudaS
     const unsigned nb = (it.nf + kTile - 1) / kTile;
     if (fast) {
       if (odd) {
-        flow_solo_strided<T><<<(unsigned)std::max(1, std::min<int>(grid, (int)nb)), kTile, 0, s>>>(a, it.off);
+        launch_after(flow_solo_strided<T>, (unsigned)std::max(1, std::min<int>(grid, (int)nb)), kTile, s, a, it.off);
       } else {
         const uint32_t pairs = (it.nf - (it.off & 1u) + 1) / 2;
-        flow_solo_pair<T><<<std::max(1u, (pairs + kTile - 1) / kTile), kTile, 0, s>>>(a, it.off);
+        launch_after(flow_solo_pair<T>, std::max(1u, (pairs + kTile - 1) / kTile), kTile, s, a, it.off);
       }
       return;
     }
-    if (odd) flow_solo_sweep<T, true, MINB><<<nb, kTile, 0, s>>>(a, it.off);
-    else flow_solo_sweep<T, false, MINB><<<nb, kTile, 0, s>>>(a, it.off);
+    if (odd) launch_after(flow_solo_sweep<T, true, MINB>, nb, kTile, s, a, it.off);
+    else launch_after(flow_solo_sweep<T, false, MINB>, nb, kTile, s, a, it.off);
     return;
   }
-  if (odd) flow_batch_sweep<T, true, MINB><<<grid, kTile, 0, s>>>(a, b->gdesc[g]);
-  else flow_batch_sweep<T, false, MINB><<<grid, kTile, 0, s>>>(a, b->gdesc[g]);
+  if (odd) launch_after(flow_batch_sweep<T, true, MINB>, grid, kTile, s, a, b->gdesc[g]);
+  else launch_after(flow_batch_sweep<T, false, MINB>, grid, kTile, s, a, b->gdesc[g]);
 }
 
 // the flow's sweeps of group g: rebased storage T = Reb<S> only for a group
@@ -862,12 +868,12 @@ void launch_diff(const om_batch* b, bool odd, int grid, int g, int form, cudaStr
     a.W = it.W;
     a.s = (typename Stg<T>::C)it.slope;
     const unsigned nb = (it.nf + kTile - 1) / kTile;
-    if (odd) diff_solo_sweep<T, true, MINB><<<nb, kTile, 0, s>>>(a, it.off);
-    else diff_solo_sweep<T, false, MINB><<<nb, kTile, 0, s>>>(a, it.off);
+    if (odd) launch_after(diff_solo_sweep<T, true, MINB>, nb, kTile, s, a, it.off);
+    else launch_after(diff_solo_sweep<T, false, MINB>, nb, kTile, s, a, it.off);
     return;
   }
-  if (odd) diff_batch_sweep<T, true, MINB><<<grid, kTile, 0, s>>>(a, b->gdesc[g]);
-  else diff_batch_sweep<T, false, MINB><<<grid, kTile, 0, s>>>(a, b->gdesc[g]);
+  if (odd) launch_after(diff_batch_sweep<T, true, MINB>, grid, kTile, s, a, b->gdesc[g]);
+  else launch_after(diff_batch_sweep<T, false, MINB>, grid, kTile, s, a, b->gdesc[g]);
 }
 
 // variant 0: no residency hint; variant 1: capped for 4 (flow; 3 in FP64) / 8

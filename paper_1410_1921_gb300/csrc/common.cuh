@@ -163,6 +163,33 @@ inline unsigned resident_grid(K kernel, unsigned nb, int threads = 256, size_t s
   return nb < r ? nb : r;
 }
 
+// Sweeps follow one another on a stream with nothing between them.  Each is
+// launched with programmatic stream serialisation: its blocks may start
+// once every block of the sweep before has started (grid_trigger), work out
+// their neighbours from arrays no sweep writes, and wait (grid_wait) for
+// that sweep to complete before they touch a population, a reference or a
+// boundary buffer.  That hides the launch, the ramp and the lookups behind
+// the tail of the sweep before: a 100-step window of both models on twenty
+// structures of ~68^3 9.59 -> 9.10 ms, on 256^3 (sweeps of 45 to 177 us) 0.6 %.
+// Every thread that goes on to touch such data passes grid_wait first, so a
+// completed sweep implies that all sweeps before it have completed.  In a
+// kernel launched without the attribute both are no-ops.
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+inline void launch_after(void (*k)(P...), unsigned grid, unsigned threads, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, k, P(args)...);  // a failure is the callers' cudaGetLastError
+}
+
 // Launch variants the autotuner chose, remembered for the life of the
 // process per (solver kind, precision, device, octave of the node count):
 // the first solver of a class times the variants, later ones reuse the choice.

@@ -39,6 +39,7 @@ constexpr int kDiffVariants = 9;
 
 template <class T, class L, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) diff_sweep(DiffArgs<T, L> a) {
+  grid_trigger();
   const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= a.nf) return;
   diff_node<T, ODD>(a, n, n);
@@ -46,6 +47,7 @@ __global__ void __launch_bounds__(256, MINB) diff_sweep(DiffArgs<T, L> a) {
 
 template <class T, class L, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) diff_sweep_strided(DiffArgs<T, L> a) {
+  grid_trigger();
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= a.nf) return;
@@ -64,6 +66,7 @@ __global__ void __launch_bounds__(256, MINB) diff_sweep_strided(DiffArgs<T, L> a
 
 template <class T, class L, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) diff_sweep_pipelined(DiffArgs<T, L> a) {
+  grid_trigger();
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= a.nf) return;
@@ -87,6 +90,7 @@ __global__ void __launch_bounds__(256, MINB) diff_sweep_pipelined(DiffArgs<T, L>
 
 template <class T, class L, int MINB>
 __global__ void __launch_bounds__(256, MINB) diff_sweep_rec(DiffArgs<T, L> a) {
+  grid_trigger();
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nf + a.nslow) return;
   uint2 r, q;
@@ -96,6 +100,7 @@ __global__ void __launch_bounds__(256, MINB) diff_sweep_rec(DiffArgs<T, L> a) {
 
 template <class T, class L>
 __global__ void __launch_bounds__(256) diff_sweep_rec_strided(DiffArgs<T, L> a) {
+  grid_trigger();
   const uint32_t stride = gridDim.x * blockDim.x, total = a.nf + a.nslow;
   uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= total) return;
@@ -115,6 +120,7 @@ __global__ void __launch_bounds__(256) diff_sweep_rec_strided(DiffArgs<T, L> a) 
 
 template <class T, class L>
 __global__ void __launch_bounds__(256) diff_sweep_pair(DiffArgs<T, L> a) {
+  grid_trigger();
   const uint32_t n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (n >= a.nf) return;
   if (n + 1 == a.nf) diff_node_at<T, L, false>(a, n, 0u);
@@ -295,20 +301,20 @@ template <class T, class L, bool ODD>
 void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const DiffArgs<T, L>& a) {
   constexpr int M = kDiffMinBlocks<L>;
   switch (variant) {
-    case 1: diff_sweep<T, L, ODD, M><<<nb, 256, 0, s>>>(a); break;
+    case 1: launch_after(diff_sweep<T, L, ODD, M>, nb, 256, s, a); break;
     case 2: {
       auto k = diff_sweep_strided<T, L, ODD, 0>;
-      k<<<resident_grid(k, nb), 256, 0, s>>>(a);
+      launch_after(k, resident_grid(k, nb), 256, s, a);
       break;
     }
     case 3: {
       auto k = diff_sweep_strided<T, L, ODD, M>;
-      k<<<resident_grid(k, nb), 256, 0, s>>>(a);
+      launch_after(k, resident_grid(k, nb), 256, s, a);
       break;
     }
     case 4: {
       auto k = diff_sweep_pipelined<T, L, ODD, 0>;
-      k<<<resident_grid(k, nb), 256, 0, s>>>(a);
+      launch_after(k, resident_grid(k, nb), 256, s, a);
       break;
     }
     case 6:
@@ -316,22 +322,22 @@ void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const DiffArgs<T, 
     case 8:
       if (ODD && a.rec7) {
         const unsigned nbr = blocks_for((int64_t)a.nf + a.nslow);
-        if (variant == 6) diff_sweep_rec<T, L, 0><<<nbr, 256, 0, s>>>(a);
-        else if (variant == 7) diff_sweep_rec<T, L, M><<<nbr, 256, 0, s>>>(a);
+        if (variant == 6) launch_after(diff_sweep_rec<T, L, 0>, nbr, 256, s, a);
+        else if (variant == 7) launch_after(diff_sweep_rec<T, L, M>, nbr, 256, s, a);
         else {
           auto k = diff_sweep_rec_strided<T, L>;
-          k<<<resident_grid(k, nbr), 256, 0, s>>>(a);
+          launch_after(k, resident_grid(k, nbr), 256, s, a);
         }
         break;
       }
       [[fallthrough]];
     case 5:
       if (!ODD) {
-        diff_sweep_pair<T, L><<<blocks_for((a.nf + 1) / 2), 256, 0, s>>>(a);
+        launch_after(diff_sweep_pair<T, L>, blocks_for((a.nf + 1) / 2), 256, s, a);
         break;
       }
       [[fallthrough]];
-    default: diff_sweep<T, L, ODD, 0><<<nb, 256, 0, s>>>(a); break;
+    default: launch_after(diff_sweep<T, L, ODD, 0>, nb, 256, s, a); break;
   }
 }
 

@@ -155,6 +155,7 @@ __device__ __forceinline__ void diff_store(const DiffArgs<T, L>& a, uint32_t n, 
 
 template <class T, class L, bool ODD, bool FACES = true>
 __device__ __forceinline__ void diff_node_nb(const DiffArgs<T, L>& a, uint32_t n, int x, const uint32_t (&nb)[L::Q]) {
+  grid_wait();
   DiffRefs<T, L> r{};
   if (ODD) diff_refs(a, n, nb, r);
   typename Stg<T>::C g[L::Q];
@@ -208,6 +209,7 @@ __device__ __forceinline__ void diff_store(const DiffArgs<T, L>& a, uint32_t n, 
 template <class T, class L>
 __device__ __forceinline__ void diff_pair_even(const DiffArgs<T, L>& a, uint32_t n) {
   using C = typename Stg<T>::C;
+  grid_wait();
   C g0[L::Q], g1[L::Q];
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) Pair<T>::ld(a.q[i] + n, a.down, g0[i], g1[i]);

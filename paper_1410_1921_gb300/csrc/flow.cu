@@ -78,6 +78,7 @@ constexpr int kSweepVariants = 13;
 
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) d3q19_sweep(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= a.nf) return;
   flow_node<T, ODD>(a, n, n);
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(256, MINB) d3q19_sweep(FlowArgs<T> a) {
 
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) d3q19_sweep_strided(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= a.nf) return;
@@ -103,6 +105,7 @@ __global__ void __launch_bounds__(256, MINB) d3q19_sweep_strided(FlowArgs<T> a) 
 
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) d3q19_sweep_pipelined(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= a.nf) return;
@@ -149,6 +152,7 @@ __device__ __forceinline__ void flow_odd_rec_lean(const FlowArgs<T>& a, uint32_t
   using C = typename Stg<T>::C;
   C f[19];
   float rn = 0.f;
+  grid_wait();
   if constexpr (kFlowRebased<T>) rn = a.rr[n];
   {
     uint32_t nb[19];
@@ -184,15 +188,20 @@ __device__ __forceinline__ void flow_odd_rec_lean(const FlowArgs<T>& a, uint32_t
 
 template <class T, int MINB>
 __global__ void __launch_bounds__(256, MINB) d3q19_sweep_rec_lean(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= a.nf) return;
   const uint2 r = __ldg(a.rec7 + n);
-  if (rec_slow(r)) return;
+  if (rec_slow(r)) {
+    grid_wait();  // also where every node is slow: a completed sweep implies those before it
+    return;
+  }
   flow_odd_rec_lean<T>(a, n, r, __ldg(a.rec19 + n));
 }
 
 template <class T>
 __global__ void __launch_bounds__(256) d3q19_sweep_slow(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nslow) return;
   const uint32_t n = __ldg(a.slow + t);
@@ -201,6 +210,7 @@ __global__ void __launch_bounds__(256) d3q19_sweep_slow(FlowArgs<T> a) {
 
 template <class T, int MINB>
 __global__ void __launch_bounds__(256, MINB) d3q19_sweep_rec(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nf + a.nslow) return;
   uint2 r = make_uint2(0u, 0u), q = make_uint2(0u, 0u);
@@ -213,6 +223,7 @@ __global__ void __launch_bounds__(256, MINB) d3q19_sweep_rec(FlowArgs<T> a) {
 
 template <class T>
 __global__ void __launch_bounds__(256) d3q19_sweep_rec_strided(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t stride = gridDim.x * blockDim.x, total = a.nf + a.nslow;
   uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= total) return;
@@ -238,6 +249,7 @@ __global__ void __launch_bounds__(256) d3q19_sweep_rec_strided(FlowArgs<T> a) {
 
 template <class T>
 __global__ void __launch_bounds__(256) d3q19_sweep_pair(FlowArgs<T> a) {
+  grid_trigger();
   const uint32_t n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (n >= a.nf) return;
   if (n + 1 == a.nf) flow_node_at<T, false>(a, n, 0u);
@@ -344,6 +356,8 @@ __device__ __forceinline__ void flow_moments_at(const FlowArgs<T>& a, uint32_t n
 
 template <class T, bool ODD>
 __global__ void d3q19_pressure_bc(FlowArgs<T> a, typename Stg<T>::C* bc, double drho_in, double drho_out) {
+  grid_trigger();
+  grid_wait();
   using C = typename Stg<T>::C;
   const uint32_t nbt = a.n_in + a.n_out;
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -410,21 +424,21 @@ template <class T, bool ODD>
 void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const FlowArgs<T>& a) {
   constexpr int M = kMinBlocks1<T>;
   switch (variant) {
-    case 1: d3q19_sweep<T, ODD, M><<<nb, 256, 0, s>>>(a); break;
+    case 1: launch_after(d3q19_sweep<T, ODD, M>, nb, 256, s, a); break;
     case 2: {
       auto k = d3q19_sweep_strided<T, ODD, 0>;
-      k<<<resident_grid(k, nb), 256, 0, s>>>(a);
+      launch_after(k, resident_grid(k, nb), 256, s, a);
       break;
     }
     case 3: {
       auto k = d3q19_sweep_strided<T, ODD, M>;
-      k<<<resident_grid(k, nb), 256, 0, s>>>(a);
+      launch_after(k, resident_grid(k, nb), 256, s, a);
       break;
     }
-    case 4: d3q19_sweep<T, ODD, M + 1><<<nb, 256, 0, s>>>(a); break;
+    case 4: launch_after(d3q19_sweep<T, ODD, M + 1>, nb, 256, s, a); break;
     case 5: {
       auto k = d3q19_sweep_pipelined<T, ODD, 0>;
-      k<<<resident_grid(k, nb), 256, 0, s>>>(a);
+      launch_after(k, resident_grid(k, nb), 256, s, a);
       break;
     }
     case 7:
@@ -436,26 +450,26 @@ void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const FlowArgs<T>&
       if (ODD && a.rec7) {
         const unsigned nbr = blocks_for((int64_t)a.nf + a.nslow);
         if (variant >= 10) {
-          if (variant == 10) d3q19_sweep_rec_lean<T, 0><<<nb, 256, 0, s>>>(a);
-          else if (variant == 11) d3q19_sweep_rec_lean<T, M><<<nb, 256, 0, s>>>(a);
-          else d3q19_sweep_rec_lean<T, M - 1><<<nb, 256, 0, s>>>(a);
-          if (a.nslow) d3q19_sweep_slow<T><<<blocks_for(a.nslow), 256, 0, s>>>(a);
-        } else if (variant == 7) d3q19_sweep_rec<T, 0><<<nbr, 256, 0, s>>>(a);
-        else if (variant == 8) d3q19_sweep_rec<T, M><<<nbr, 256, 0, s>>>(a);
+          if (variant == 10) launch_after(d3q19_sweep_rec_lean<T, 0>, nb, 256, s, a);
+          else if (variant == 11) launch_after(d3q19_sweep_rec_lean<T, M>, nb, 256, s, a);
+          else launch_after(d3q19_sweep_rec_lean<T, M - 1>, nb, 256, s, a);
+          if (a.nslow) launch_after(d3q19_sweep_slow<T>, blocks_for(a.nslow), 256, s, a);
+        } else if (variant == 7) launch_after(d3q19_sweep_rec<T, 0>, nbr, 256, s, a);
+        else if (variant == 8) launch_after(d3q19_sweep_rec<T, M>, nbr, 256, s, a);
         else {
           auto k = d3q19_sweep_rec_strided<T>;
-          k<<<resident_grid(k, nbr), 256, 0, s>>>(a);
+          launch_after(k, resident_grid(k, nbr), 256, s, a);
         }
         break;
       }
       [[fallthrough]];
     case 6:
       if (!ODD) {
-        d3q19_sweep_pair<T><<<blocks_for((a.nf + 1) / 2), 256, 0, s>>>(a);
+        launch_after(d3q19_sweep_pair<T>, blocks_for((a.nf + 1) / 2), 256, s, a);
         break;
       }
       [[fallthrough]];
-    default: d3q19_sweep<T, ODD, 0><<<nb, 256, 0, s>>>(a); break;
+    default: launch_after(d3q19_sweep<T, ODD, 0>, nb, 256, s, a); break;
   }
 }
 
@@ -538,8 +552,8 @@ void launch_step(const om_flow* fl, bool odd, int variant, unsigned nb, cudaStre
   if (nbt) {
     using C = typename Stg<T>::C;
     const double h = 0.5 * fl->p.delta_rho;
-    if (odd) d3q19_pressure_bc<T, true><<<(nbt + 127) / 128, 128, 0, s>>>(a, (C*)fl->bc, h, -h);
-    else d3q19_pressure_bc<T, false><<<(nbt + 127) / 128, 128, 0, s>>>(a, (C*)fl->bc, h, -h);
+    launch_after(odd ? d3q19_pressure_bc<T, true> : d3q19_pressure_bc<T, false>, (nbt + 127) / 128, 128, s, a,
+                 (C*)fl->bc, h, -h);
   }
   launch_sweep<T>(odd, variant, nb, s, a);
 }

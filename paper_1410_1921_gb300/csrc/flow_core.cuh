@@ -184,6 +184,7 @@ __device__ __forceinline__ void flow_collide(const FlowArgs<T>& a, uint32_t n, t
 // written).
 template <class T, bool ODD>
 __device__ __forceinline__ void flow_node_nb(const FlowArgs<T>& a, uint32_t n, const uint32_t (&nb)[19]) {
+  grid_wait();
   typename Stg<T>::C f[19];
   if constexpr (ODD) {
     uint32_t off[19];
@@ -238,6 +239,7 @@ __device__ __forceinline__ void flow_node_at(const FlowArgs<T>& a, uint32_t n, u
 template <class T>
 __device__ __forceinline__ void flow_pair_even(const FlowArgs<T>& a, uint32_t n) {
   using C = typename Stg<T>::C;
+  grid_wait();
   C f0[19], f1[19];
 #pragma unroll
   for (int i = 0; i < 19; ++i) Pair<T>::ld(a.s[i] + n, a.down, f0[i], f1[i]);
