@@ -99,7 +99,9 @@ typedef struct {
    * neighbour records, one thread per node / capped / on a resident grid,
    * even steps as 6; 10/11/12 odd steps from the records holding only the
    * populations across the collision, uncapped / capped / capped tighter,
-   * even steps as 6); larger values clamp to 12.  A batch (om_batch_create)
+   * even steps as 6; 13/14 odd steps with the slot offsets parked in shared
+   * memory, neighbours from the column map / the records, even steps as 6);
+   * larger values clamp to 14.  A batch (om_batch_create)
    * takes 0..3: 0/1 one thread per node without/with a register cap, 2 as 1
    * with each structure large enough for a group of its own in the forms
    * of 2 (odd) and 6 (even), 3 as 1 with each such structure in this

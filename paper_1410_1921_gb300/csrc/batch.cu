@@ -118,6 +118,54 @@ __device__ __forceinline__ void diff_group_tile(const DiffArgs<T>& a, const Grou
   diff_node<T, ODD>(b, it.off + ln, ln);
 }
 
+// The odd steps of tile w with the slot offsets parked in shared memory
+// (flow_node_parked, diff_node_parked)
+template <class T>
+__device__ __forceinline__ void flow_group_tile_parked(const FlowArgs<T>& a, const GroupDesc& g, int w, uint32_t* parked) {
+  const int k = group_item(g, w);
+  const GroupItem& it = g.it[k];
+  const uint32_t ln = (uint32_t)(w - g.tile0[k]) * kTile + threadIdx.x;
+  if (ln >= it.nf) return;
+  uint32_t nb[19];
+  q19_neighbours(it.col, it.nx, it.ny, it.nz, it.W, 1, __ldg(it.coord + ln), nb);
+  flow_node_parked(a, it.off + ln, nb, parked);
+}
+
+template <class T>
+__device__ __forceinline__ void diff_group_tile_parked(const DiffArgs<T>& a, const GroupDesc& g, int w, uint32_t* parked) {
+  const int k = group_item(g, w);
+  const GroupItem& it = g.it[k];
+  const uint32_t ln = (uint32_t)(w - g.tile0[k]) * kTile + threadIdx.x;
+  if (ln >= it.nf) return;
+  DiffArgs<T> b = a;
+  b.nx = it.nx;
+  b.s = (typename Stg<T>::C)it.slope;
+  b.col = it.col;
+  b.ny = it.ny;
+  b.nz = it.nz;
+  b.W = it.W;
+  uint32_t nb[7];
+  int x = 0;
+  diff_neighbours(b, __ldg(it.coord + ln), nb, x);
+  diff_node_parked(b, it.off + ln, x, nb, parked);
+}
+
+template <class T, int MINB>
+__global__ void __launch_bounds__(kTile, MINB) flow_batch_parked(FlowArgs<T> a, const __grid_constant__ GroupDesc g) {
+  grid_trigger();
+  __shared__ uint32_t parked[18 * kParkStride];
+  const int nw = g.tile0[g.n];
+  for (int w = blockIdx.x; w < nw; w += gridDim.x) flow_group_tile_parked(a, g, w, parked + threadIdx.x);
+}
+
+template <class T, int MINB>
+__global__ void __launch_bounds__(kTile, MINB) diff_batch_parked(DiffArgs<T> a, const __grid_constant__ GroupDesc g) {
+  grid_trigger();
+  __shared__ uint32_t parked[6 * kDiffParkStride];
+  const int nw = g.tile0[g.n];
+  for (int w = blockIdx.x; w < nw; w += gridDim.x) diff_group_tile_parked(a, g, w, parked + threadIdx.x);
+}
+
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(kTile, MINB) flow_batch_sweep(FlowArgs<T> a, const __grid_constant__ GroupDesc g) {
   grid_trigger();
@@ -807,7 +855,8 @@ void launch_flow_t(const om_batch* b, bool odd, int grid, int g, int form, cudaS
     else launch_after(flow_solo_sweep<T, false, MINB>, nb, kTile, s, a, it.off);
     return;
   }
-  if (odd) launch_after(flow_batch_sweep<T, true, MINB>, grid, kTile, s, a, b->gdesc[g]);
+  if (odd && MINB > 0) launch_after(flow_batch_parked<T, (sizeof(T) == 8 ? 4 : 6)>, grid, kTile, s, a, b->gdesc[g]);
+  else if (odd) launch_after(flow_batch_sweep<T, true, MINB>, grid, kTile, s, a, b->gdesc[g]);
   else launch_after(flow_batch_sweep<T, false, MINB>, grid, kTile, s, a, b->gdesc[g]);
 }
 
@@ -872,12 +921,14 @@ void launch_diff(const om_batch* b, bool odd, int grid, int g, int form, cudaStr
     else launch_after(diff_solo_sweep<T, false, MINB>, nb, kTile, s, a, it.off);
     return;
   }
-  if (odd) launch_after(diff_batch_sweep<T, true, MINB>, grid, kTile, s, a, b->gdesc[g]);
+  if (odd && MINB > 0) launch_after(diff_batch_parked<T, 6>, grid, kTile, s, a, b->gdesc[g]);
+  else if (odd) launch_after(diff_batch_sweep<T, true, MINB>, grid, kTile, s, a, b->gdesc[g]);
   else launch_after(diff_batch_sweep<T, false, MINB>, grid, kTile, s, a, b->gdesc[g]);
 }
 
-// variant 0: no residency hint; variant 1: capped for 4 (flow; 3 in FP64) / 8
-// (diffusion) CTAs per SM; variant 2 (flow): as 1, with the solo groups in
+// variant 0: no residency hint; variant 1: even steps capped for 4 (flow; 3 in
+// FP64) / 8 (diffusion) CTAs per SM, odd steps with the slot offsets parked
+// in shared memory, 6 CTAs per SM (flow in FP64: 4); variant 2 (flow): as 1, with the solo groups in
 // the single-structure solver's fastest forms (flow_solo_strided / _pair);
 // variant 3 (flow): as 1, with each solo group in the single-structure
 // solver's own sweeps, the variants tuned for its size

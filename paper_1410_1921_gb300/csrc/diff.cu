@@ -34,8 +34,12 @@ namespace om {
 // steps as variant 0; 6, 7, 8 = odd steps from the neighbour records with
 // the slow nodes in the same grid (the flow sweep's variants 7, 8, 9: one
 // thread per node, capped, and a resident grid loading the next node's
-// records ahead), even steps as variant 5.  Without records 6-8 run as 5.
-constexpr int kDiffVariants = 9;
+// records ahead), even steps as variant 5; 9 = odd steps with the slot
+// offsets parked in shared memory (diff_node_parked in diff_core.cuh), from
+// the records, even steps as variant 5.  5.76 M nodes, odd + even: FP32 D3Q19
+// 457 us in variant 6, 363 in 9; D3Q7 139 us, 134.  Without records 6-9 run
+// as 5.
+constexpr int kDiffVariants = 10;
 
 template <class T, class L, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) diff_sweep(DiffArgs<T, L> a) {
@@ -116,6 +120,36 @@ __global__ void __launch_bounds__(256) diff_sweep_rec_strided(DiffArgs<T, L> a) 
     r = rn;
     q = qn;
   }
+}
+
+// Odd step with the slot offsets parked in shared memory (diff_node_parked):
+// the nodes with records, one thread each; the slow nodes as their own
+// launch, whose x-face cases then set no register budget here.
+template <class T, class L, int MINB>
+__global__ void __launch_bounds__(256, MINB) diff_sweep_parked(DiffArgs<T, L> a) {
+  grid_trigger();
+  __shared__ uint32_t parked[(L::Q - 1) * kDiffParkStride];
+  const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= a.nf) return;
+  uint2 r, q;
+  diff_rec_load<L>(a.rec7, a.rec19, n, a.nf, r, q);
+  if (rec_slow(r)) {
+    grid_wait();  // also where every node is slow: a completed sweep implies those before it
+    return;
+  }
+  uint32_t nb[L::Q];
+  if constexpr (L::Q == 19) rec_neighbours19(r, q, n, nb);
+  else rec_axis<L::Q>(r, n, nb);
+  diff_node_parked<T, L, false>(a, n, 0, nb, parked + threadIdx.x);
+}
+
+template <class T, class L>
+__global__ void __launch_bounds__(256) diff_sweep_slow(DiffArgs<T, L> a) {
+  grid_trigger();
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= a.nslow) return;
+  const uint32_t n = __ldg(a.slow + t);
+  diff_node_at<T, L, true>(a, n, __ldg(a.coord + n));
 }
 
 template <class T, class L>
@@ -328,6 +362,14 @@ void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const DiffArgs<T, 
           auto k = diff_sweep_rec_strided<T, L>;
           launch_after(k, resident_grid(k, nbr), 256, s, a);
         }
+        break;
+      }
+      [[fallthrough]];
+    case 9:
+      if (ODD && a.rec7) {
+        constexpr int B = L::Q == 19 && sizeof(T) == 8 ? 4 : 6;
+        launch_after(diff_sweep_parked<T, L, B>, nb, 256, s, a);
+        if (a.nslow) launch_after(diff_sweep_slow<T, L>, blocks_for(a.nslow), 256, s, a);
         break;
       }
       [[fallthrough]];

@@ -221,6 +221,64 @@ __device__ __forceinline__ void diff_pair_even(const DiffArgs<T, L>& a, uint32_t
   for (int i = 0; i < L::Q; ++i) Pair<T>::st(a.q[L::opp(i)] + n, g0[i], g1[i], a.up);
 }
 
+// Odd step of diff_node_nb with the slot offsets parked in shared memory
+// while the node relaxes (as flow_node_parked in flow_core.cuh): neither the
+// slot addresses nor the neighbours' reference concentrations are held, the
+// references are gathered again for the stores (they hit L1).
+constexpr int kDiffParkStride = 256;
+template <class T, class L, bool FACES = true>
+__device__ __forceinline__ void diff_node_parked(const DiffArgs<T, L>& a, uint32_t n, int x, const uint32_t (&nb)[L::Q],
+                                                 uint32_t* parked) {
+  using S = Stg<T>;
+  using C = typename S::C;
+  grid_wait();
+  const uint32_t P = (uint32_t)(a.q[1] - a.q[0]);
+  C g[L::Q], rn = 0;
+  if constexpr (kRebased<T>) rn = (C)a.cr[n];
+  g[0] = S::ld(a.q[0] + n, a.down);
+#pragma unroll
+  for (int i = 1; i < L::Q; ++i) {
+    const uint32_t o = (uint32_t)L::opp(i), src = nb[o];
+    const bool inlet = FACES && from_inlet<L>(i, x), outlet = FACES && from_outlet<L>(i, x, a.nx);
+    const bool there = src != kNoNode && !inlet && !outlet;
+    const uint32_t off = there ? o * P + src : (uint32_t)i * P + n;
+    parked[(i - 1) * kDiffParkStride] = off;
+    const C v = S::ld(a.q[0] + off, a.down), w = C(L::w(i));
+    if constexpr (kRebased<T>) {
+      if (inlet) g[i] = -v + C(2) * w * ((C)a.cin - rn);
+      else if (outlet) g[i] = -v + C(2) * w * ((C)a.cout - rn);
+      else if (there) g[i] = v + w * ((C)a.cr[src] - rn);
+      else g[i] = v;
+    } else {
+      if (inlet) g[i] = -v - w * a.s;
+      else if (outlet) g[i] = -v + w * a.s;
+      else if (there) g[i] = v - w * C(L::e(i, 0)) * a.s;
+      else g[i] = v;
+    }
+  }
+  asm volatile("" ::: "memory");  // the offsets are read back, not kept
+  diff_relax<L>(g, a.omega[n]);
+  S::st(a.q[0] + n, g[0], a.up);
+#pragma unroll
+  for (int i = 1; i < L::Q; ++i) {
+    const uint32_t to = parked[(L::opp(i) - 1) * kDiffParkStride];
+    const uint32_t dst = to - (uint32_t)i * P;  // below P: another node's slot, of node dst
+    const bool outlet = FACES && L::e(i, 0) == 1 && x == a.nx - 1, inlet = FACES && L::e(i, 0) == -1 && x == 0;
+    const C w = C(L::w(i));
+    C v = g[i];
+    if constexpr (kRebased<T>) {
+      if (outlet) v = -g[i] + C(2) * w * ((C)a.cout - rn);
+      else if (inlet) v = -g[i] + C(2) * w * ((C)a.cin - rn);
+      else if (dst < P) v = g[i] + w * (rn - (C)a.cr[dst]);
+    } else {
+      if (outlet) v = -g[i] + w * a.s;
+      else if (inlet) v = -g[i] - w * a.s;
+      else if (dst < P) v = g[i] - w * C(L::e(i, 0)) * a.s;
+    }
+    S::st(a.q[0] + to, v, a.up);
+  }
+}
+
 // diff_node_nb after the neighbour lookup of the node's coordinates c
 template <class T, class L, bool ODD>
 __device__ __forceinline__ void diff_node_at(const DiffArgs<T, L>& a, uint32_t n, uint32_t c) {

@@ -67,14 +67,24 @@ namespace om {
 //   9  variant 7 on a resident grid whose threads stride over the nodes
 //      (then the slow list) and load the next node's records before
 //      updating the current one.
-//   Without records (a box beyond their fields) 7-9 run as 6.
+//   13 odd steps with the slot offsets parked in shared memory while the
+//      node collides, neighbours from the column map (flow_node_parked in
+//      flow_core.cuh), even steps as variant 6.  5.76 M nodes, FP32: odd step
+//      177 us in variant 2, 168 so;
+//   14 the same with the neighbours from the records, the slow nodes in the
+//      same grid.  FP16 rebased storage: odd + even 324 us in variant 9,
+//      282 so.
+//   Without records (a box beyond their fields) 7-9 and 14 run as 6.
 // (Odd steps of two nodes per thread, a grid apart, with both lookups and
 // all 38 loads issued before either update, were measured slower than
 // variant 2: the registers they need halve the resident threads.)
 template <class T>
 constexpr int kMinBlocks1 = sizeof(T) == 8 ? 3 : 4;
+// resident blocks of 256 with parked offsets: 40 registers (FP64: 64, which its 19 doubles need)
+template <class T>
+constexpr int kParkBlocks = sizeof(T) == 8 ? 4 : 6;
 
-constexpr int kSweepVariants = 13;
+constexpr int kSweepVariants = 15;
 
 template <class T, bool ODD, int MINB>
 __global__ void __launch_bounds__(256, MINB) d3q19_sweep(FlowArgs<T> a) {
@@ -245,6 +255,32 @@ __global__ void __launch_bounds__(256) d3q19_sweep_rec_strided(FlowArgs<T> a) {
     r = rn;
     q = qn;
   }
+}
+
+// Odd step with the slot offsets parked in shared memory (flow_node_parked),
+// one thread per node; REC: neighbours from the records, with the slow nodes
+// at the end of the grid, else from the column map.
+template <class T, int MINB, bool REC>
+__global__ void __launch_bounds__(256, MINB) d3q19_sweep_parked(FlowArgs<T> a) {
+  grid_trigger();
+  __shared__ uint32_t parked[18 * kParkStride];
+  uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t nb[19];
+  if (REC) {
+    if (n >= a.nf + a.nslow) return;
+    if (n < a.nf) {
+      const uint2 r = __ldg(a.rec7 + n), q = __ldg(a.rec19 + n);
+      if (rec_slow(r)) return;  // at the end of the grid
+      rec_neighbours19(r, q, n, nb);
+    } else {
+      n = __ldg(a.slow + (n - a.nf));
+      flow_neighbours(a, __ldg(a.coord + n), nb);
+    }
+  } else {
+    if (n >= a.nf) return;
+    flow_neighbours(a, __ldg(a.coord + n), nb);
+  }
+  flow_node_parked(a, n, nb, parked + threadIdx.x);
 }
 
 template <class T>
@@ -460,6 +496,18 @@ void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const FlowArgs<T>&
           auto k = d3q19_sweep_rec_strided<T>;
           launch_after(k, resident_grid(k, nbr), 256, s, a);
         }
+        break;
+      }
+      [[fallthrough]];
+    case 13:
+      if (ODD) {
+        launch_after(d3q19_sweep_parked<T, kParkBlocks<T>, false>, nb, 256, s, a);
+        break;
+      }
+      [[fallthrough]];
+    case 14:
+      if (ODD && a.rec7) {
+        launch_after(d3q19_sweep_parked<T, kParkBlocks<T>, true>, blocks_for((int64_t)a.nf + a.nslow), 256, s, a);
         break;
       }
       [[fallthrough]];

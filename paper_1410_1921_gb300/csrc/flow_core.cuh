@@ -225,6 +225,48 @@ __device__ __forceinline__ void flow_node_nb(const FlowArgs<T>& a, uint32_t n, c
   }
 }
 
+// Odd step of flow_node_nb with the 18 slot offsets parked in shared memory
+// while the node collides: parked[k * kParkStride] is this thread's k-th
+// word.  What bounds the odd step is the latency of its dependent chain
+// (record or coordinates, column words, populations), so resident warps
+// count: without the offsets 40 registers do instead of 80 (128 for rebased
+// storage), six blocks of 256 instead of three (two).  The references of
+// rebased storage are gathered again after the collision (they hit L1).
+constexpr int kParkStride = 256;
+template <class T>
+__device__ __forceinline__ void flow_node_parked(const FlowArgs<T>& a, uint32_t n, const uint32_t (&nb)[19],
+                                                 uint32_t* parked) {
+  using C = typename Stg<T>::C;
+  grid_wait();
+  C f[19];
+  float rn = 0.f;
+  if constexpr (kFlowRebased<T>) rn = a.rr[n];
+  f[0] = Stg<T>::ld(a.s[0] + n, a.down);
+#pragma unroll
+  for (int i = 1; i < 19; ++i) {
+    const uint32_t o = (uint32_t)q19_opp(i), src = nb[o];
+    const uint32_t off = src != kNoNode ? o * a.P + src : (uint32_t)i * a.P + n;
+    parked[(i - 1) * kParkStride] = off;
+    f[i] = Stg<T>::ld(a.s[0] + off, a.down);
+    if constexpr (kFlowRebased<T>)
+      if (src != kNoNode) f[i] += (float)q19_w(i) * (a.rr[src] - rn);
+  }
+  asm volatile("" ::: "memory");  // the offsets are read back, not kept
+  flow_collide(a, n, f);
+  order_after(f[16], f[17]);
+  Stg<T>::st(a.s[0] + n, f[0], a.up);
+#pragma unroll
+  for (int i = 1; i < 19; ++i) {
+    const uint32_t to = parked[(q19_opp(i) - 1) * kParkStride];
+    C v = f[i];
+    if constexpr (kFlowRebased<T>) {
+      const uint32_t dst = to - (uint32_t)i * a.P;  // below P: another node's slot, of node dst
+      if (dst < a.P) v -= (float)q19_w(i) * (a.rr[dst] - rn);
+    }
+    Stg<T>::st(a.s[0] + to, v, a.up);
+  }
+}
+
 // flow_node_nb after the neighbour lookup of the node's coordinates c
 template <class T, bool ODD>
 __device__ __forceinline__ void flow_node_at(const FlowArgs<T>& a, uint32_t n, uint32_t c) {
