@@ -48,6 +48,7 @@ struct SplitMix64 {
 struct Ball {
   double c[3];
   double r;
+  double v;  // ball_volume(r)
 };
 
 double ball_volume(double r) { return (4.0 * kPi / 3.0) * (r * r * r); }
@@ -77,7 +78,7 @@ struct Placer {
   // uniform grid of cells, each at least one maximal diameter wide
   int gx = 1, gy = 1, gz = 1;
   double hx = 1, hy = 1, hz = 1;
-  std::vector<std::vector<int32_t>> cells;
+  std::vector<std::vector<Ball>> cells;  // copies, so that a cell's balls lie together
   int64_t trials = 0;
 
   void init(uint64_t seed) {
@@ -110,7 +111,7 @@ struct Placer {
 
   // tolerance and overlap-requirement test of a trial against placed balls
   bool acceptable(const Ball& t, bool must_touch) const {
-    const double vt = ball_volume(t.r);
+    const double vt = t.v;
     bool touched = false;
     const int ix = cell_of(t.c[0], hx, gx), iy = cell_of(t.c[1], hy, gy), iz = cell_of(t.c[2], hz, gz);
     int ys[3], zs[3], ny = 0, nz = 0;
@@ -122,22 +123,26 @@ struct Placer {
     for (int x = std::max(0, ix - 1); x <= std::min(gx - 1, ix + 1); ++x)
       for (int a = 0; a < ny; ++a)
         for (int b = 0; b < nz; ++b)
-          for (int32_t k : cells[((size_t)x * gy + ys[a]) * gz + zs[b]]) {
-            const Ball& s = balls[k];
+          for (const Ball& s : cells[((size_t)x * gy + ys[a]) * gz + zs[b]]) {
+            // most balls of the cells are out of reach: then the overlap is 0 and changes nothing.
+            // Clear by more than any rounding of the distance, without its square root
+            const double reach = (t.r + s.r) * (1.0 + 1e-9);
             const double dx = t.c[0] - s.c[0];
+            if (dx > reach || -dx > reach) continue;
             const double dy = periodic_gap(t.c[1] - s.c[1], dom.ny);
             const double dz = periodic_gap(t.c[2] - s.c[2], dom.nz);
-            const double dist = std::sqrt(dx * dx + dy * dy + dz * dz);
-            const double v = overlap_volume(t.r, s.r, dist);
+            const double d2 = dx * dx + dy * dy + dz * dz;
+            if (d2 > reach * reach) continue;
+            const double v = overlap_volume(t.r, s.r, std::sqrt(d2));
             if (v > 0.0) touched = true;
-            if (v / vt > p.overlap_tol || v / ball_volume(s.r) > p.overlap_tol) return false;
+            if (v / vt > p.overlap_tol || v / s.v > p.overlap_tol) return false;
           }
     return touched || !must_touch;
   }
 
   void add(const Ball& b) {
     const int ix = cell_of(b.c[0], hx, gx), iy = cell_of(b.c[1], hy, gy), iz = cell_of(b.c[2], hz, gz);
-    cells[((size_t)ix * gy + iy) * gz + iz].push_back((int32_t)balls.size());
+    cells[((size_t)ix * gy + iy) * gz + iz].push_back(b);
     balls.push_back(b);
   }
 
@@ -153,6 +158,7 @@ struct Placer {
       t.c[1] = rng.uniform() * dom.ny;
       t.c[2] = rng.uniform() * dom.nz;
       t.r = 0.5 * (draw_diameter() / dom.dx_nm);
+      t.v = ball_volume(t.r);
       if (first || acceptable(t, must_touch)) {
         add(t);
         return true;
@@ -351,28 +357,35 @@ om_status reconstruct_impl(uint64_t seed, const om_domain& d, const om_recon_par
   std::vector<unsigned long long> cnt;
   while (kstop < 0 && !infeasible) {
     const double need = p.porosity * (double)N - (double)covered;
-    int64_t chunk = (int64_t)std::ceil(1.5 * std::max(0.0, need) / vmean) + 16;
+    // about what is needed: every sphere placed beyond the last one is wasted (serial) work, and a
+    // second, small batch costs one round trip
+    int64_t chunk = (int64_t)std::ceil(1.15 * std::max(0.0, need) / vmean) + 16;
     chunk = std::min<int64_t>(chunk, 1 << 18);
     const int k0 = (int)pl.balls.size();
-    for (int64_t i = 0; i < chunk; ++i)
-      if (!pl.place_next()) {
-        infeasible = true;
-        break;
-      }
-    const int k1 = (int)pl.balls.size();
-    if (k1 == k0) break;
-    host_balls.resize(k1 - k0);
-    for (int k = k0; k < k1; ++k) host_balls[k - k0] = to_dev(pl.balls[k], d);
     StreamBuf batch(s);
     size_t at = 0;
-    OM_TRY(batch.alloc((size_t)(k1 - k0) * (sizeof(DevBall) + sizeof(unsigned long long)) + 512));
-    DevBall* dballs = carve<DevBall>(batch.p, &at, k1 - k0);
-    unsigned long long* dcnt = carve<unsigned long long>(batch.p, &at, k1 - k0);
-    OM_CUDA(cudaMemcpyAsync(dballs, host_balls.data(), sizeof(DevBall) * (k1 - k0), cudaMemcpyHostToDevice, s));
-    OM_CUDA(cudaMemsetAsync(dcnt, 0, sizeof(unsigned long long) * (k1 - k0), s));
-    // about 16 blocks for each of the 1216 that are resident, so that large balls do not trail
-    const int nb = k1 - k0, split = std::max(1, std::min(64, 16 * 1216 / nb));
-    raster_balls<<<dim3((unsigned)nb, (unsigned)split), 256, 0, s>>>(dballs, k0, d.nx, d.ny, d.nz, owner);
+    OM_TRY(batch.alloc((size_t)chunk * (sizeof(DevBall) + sizeof(unsigned long long)) + 512));
+    DevBall* dballs = carve<DevBall>(batch.p, &at, chunk);
+    unsigned long long* dcnt = carve<unsigned long long>(batch.p, &at, chunk);
+    host_balls.resize(chunk);
+    // placed in a few parts, each rasterised while the host places the next
+    const int64_t part = std::max<int64_t>(64, (chunk + 3) / 4);
+    int done = k0;  // balls handed to the device
+    for (int64_t i = 0; i < chunk && !infeasible; ++i) {
+      infeasible = !pl.place_next();
+      const int k = (int)pl.balls.size(), n = k - done;
+      if (n == 0 || (n < part && i + 1 < chunk && !infeasible)) continue;
+      for (int j = done; j < k; ++j) host_balls[j - k0] = to_dev(pl.balls[j], d);
+      OM_CUDA(cudaMemcpyAsync(dballs + (done - k0), host_balls.data() + (done - k0), sizeof(DevBall) * n,
+                              cudaMemcpyHostToDevice, s));
+      // about 16 blocks for each of the 1216 that are resident, so that large balls do not trail
+      const int split = std::max(1, std::min(64, 16 * 1216 / n));
+      raster_balls<<<dim3((unsigned)n, (unsigned)split), 256, 0, s>>>(dballs + (done - k0), done, d.nx, d.ny, d.nz, owner);
+      done = k;
+    }
+    const int k1 = (int)pl.balls.size(), nb = k1 - k0;
+    if (nb == 0) break;
+    OM_CUDA(cudaMemsetAsync(dcnt, 0, sizeof(unsigned long long) * nb, s));
     const size_t smem = nb <= kCountSlots ? sizeof(unsigned int) * (size_t)nb : 0;
     OM_CUDA(cudaFuncSetAttribute(count_first_cover, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(unsigned int) * kCountSlots));
