@@ -536,6 +536,7 @@ om_status diff_observe_t(om_diff* df, double* out, bool with_dl, cudaStream_t s)
 
 template <class T, class L>
 om_status diff_extrapolate_t(om_diff* df, double f, cudaStream_t s) {
+  df->observed = false;
   if (df->ns->nf == 0 || !df->dprev) return OM_OK;
   DiffArgs<T, L> a = diff_args<T, L>(df);
   diff_extrapolate<T, L><<<blocks_for(a.nf), 256, 0, s>>>(a, df->prev, df->dprev, f);
@@ -621,7 +622,12 @@ om_status diff_rebase_t(om_diff* df, cudaStream_t s) {
 
 // with_dl: out[4] = sum D_L too (else 0)
 om_status diff_observe_any(om_diff* df, double* out, bool with_dl, cudaStream_t s) {
-  OM_DIFF_DISPATCH(df, diff_observe_t, df, out, with_dl, s);
+  auto go = [&]() -> om_status { OM_DIFF_DISPATCH(df, diff_observe_t, df, out, with_dl, s); };
+  df->observed = false;
+  OM_TRY(go());
+  std::copy(out, out + 5, df->last);
+  df->observed = true;
+  return OM_OK;
 }
 
 }  // namespace
@@ -680,11 +686,12 @@ extern "C" om_status om_diff_create(const om_nodeset* ns, const float* d_nm_dev,
   auto tune = [&]() -> om_status { OM_DIFF_DISPATCH(df, diff_tune_t, df, s); };
   if (p->variant >= 0) df->var[0] = df->var[1] = std::min(p->variant, kDiffVariants - 1);
   st = setup();
-  if (st == OM_OK) st = init();
-  if (st == OM_OK && p->variant < 0) {
-    st = tune();
-    if (st == OM_OK) st = init();  // back to the linear profile
+  if (st == OM_OK && p->variant < 0 &&
+      !tuned_lookup(df->q == 19 ? kTuneDiff19 : kTuneDiff7, p->precision, ns->nf, df->var)) {
+    st = init();  // the sweeps are timed from the linear profile
+    if (st == OM_OK) st = tune();
   }
+  if (st == OM_OK) st = init();
   if (st == OM_OK) {
     double o[5];
     st = diff_observe_any(df, o, false, s);
@@ -700,6 +707,7 @@ extern "C" om_status om_diff_create(const om_nodeset* ns, const float* d_nm_dev,
 extern "C" om_status om_diff_step(om_diff* df, int64_t nsteps, void* stream) {
   if (!df || nsteps < 0) return fail(OM_EINVAL, "om_diff_step: bad argument");
   cudaStream_t s = as_stream(stream);
+  if (nsteps > 0) df->observed = false;
   OM_DIFF_DISPATCH(df, diff_steps_t, df, nsteps, s);
 }
 
@@ -719,7 +727,8 @@ extern "C" om_status om_diff_solve(om_diff* df, double* D_eff_lattice, om_run_in
   OM_CUDA(cudaEventCreate(&e0));
   OM_CUDA(cudaEventCreate(&e1));
   double o[5];
-  OM_TRY(diff_observe_any(df, o, false, s));
+  if (df->observed) std::copy(df->last, df->last + 5, o);
+  else OM_TRY(diff_observe_any(df, o, false, s));
   double sj_prev = o[0];
   const int64_t t0 = df->t;
   OM_CUDA(cudaEventRecord(e0, s));
@@ -791,6 +800,7 @@ extern "C" om_status om_diff_set_populations(om_diff* df, const double* g_dev, v
   if (!df || !g_dev) return fail(OM_EINVAL, "om_diff_set_populations: null pointer");
   cudaStream_t s = as_stream(stream);
   df->t = 0;
+  df->observed = false;
   auto imp = [&]() -> om_status { OM_DIFF_DISPATCH(df, diff_import_t, df, g_dev, 0, s); };
   OM_TRY(imp());
   double o[5];
@@ -801,6 +811,7 @@ extern "C" om_status om_diff_init_concentration(om_diff* df, const float* c_dev,
                                                 void* stream) {
   if (!df || !c_dev || stride < 1) return fail(OM_EINVAL, "om_diff_init_concentration: bad argument");
   cudaStream_t s = as_stream(stream);
+  df->observed = false;
   auto init = [&]() -> om_status { OM_DIFF_DISPATCH(df, diff_init_c_t, df, c_dev, stride, from_linear, s); };
   OM_TRY(init());
   double o[5];

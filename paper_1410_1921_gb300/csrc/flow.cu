@@ -674,16 +674,15 @@ om_status flow_steps_t(om_flow* fl, int64_t nsteps, cudaStream_t s) {
 // Autotuner: time every launch variant of both sweeps on this node set
 // (6 even/odd pairs each after a warm-up pair) and keep the fastest per
 // parity; a node set of a size class tuned before in this process reuses
-// that choice.  Runs from the rest state and puts the rest state back.
+// that choice.  Times from the rest state; the caller sets the state after.
 template <class T>
 om_status flow_tune_t(om_flow* fl, cudaStream_t s) {
   if (fl->ns->nf == 0) return OM_OK;
   FlowArgs<T> a = flow_args<T>(fl);
-  bool timed = false;
-  OM_TRY(flow_tuned_variants<T>(a, fl->p.precision, flow_var<T>(fl), s, &timed));
-  if (timed) d3q19_rest<T><<<blocks_for(a.nf), 256, 0, s>>>(a);
+  if (tuned_lookup(kFlowRebased<T> ? kTuneFlowReb : kTuneFlow, fl->p.precision, a.nf, flow_var<T>(fl))) return OM_OK;
+  d3q19_rest<T><<<blocks_for(a.nf), 256, 0, s>>>(a);
   OM_CUDA(cudaGetLastError());
-  return OM_OK;
+  return flow_tuned_variants<T>(a, fl->p.precision, flow_var<T>(fl), s, nullptr);
 }
 
 template <class T>
@@ -774,6 +773,7 @@ om_status flow_enter_rebased_s(om_flow* fl, cudaStream_t s) {
 }
 om_status flow_enter_rebased(om_flow* fl, cudaStream_t s) {
   if (fl->reb || !fl->rr || (fl->t & 1)) return OM_OK;
+  fl->observed = false;
   switch (fl->p.precision) {
     case OM_F32: return flow_enter_rebased_s<float>(fl, s);
     case OM_F16DEV: return flow_enter_rebased_s<__half>(fl, s);
@@ -787,7 +787,12 @@ size_t storage_bytes(int prec) {
 }
 
 om_status flow_observe_any(om_flow* fl, double* out, cudaStream_t s) {
-  OM_FLOW_DISPATCH(fl, flow_observe_t, fl, out, s);
+  auto go = [&]() -> om_status { OM_FLOW_DISPATCH(fl, flow_observe_t, fl, out, s); };
+  fl->observed = false;
+  OM_TRY(go());
+  std::copy(out, out + 4, fl->last);
+  fl->observed = true;
+  return OM_OK;
 }
 
 }  // namespace
@@ -866,19 +871,18 @@ extern "C" om_status om_flow_create(const om_nodeset* ns, const om_flow_params* 
   auto tune = [&]() -> om_status { OM_FLOW_DISPATCH(fl, flow_tune_t, fl, s); };
   if (p->variant >= 0)
     fl->var[0] = fl->var[1] = fl->varr[0] = fl->varr[1] = std::min(p->variant, kSweepVariants - 1);
-  st = rest();
-  if (st == OM_OK && p->variant < 0) st = tune();
-  if (st == OM_OK && p->variant < 0 && fl->rr) {  // and the rebased mode's kernels, from rest
-    fl->reb = true;
-    st = rest();
-    if (st == OM_OK) st = tune();
-    fl->reb = false;
-    if (st == OM_OK) st = rest();
+  if (p->variant < 0) {
+    st = tune();
+    if (st == OM_OK && fl->rr) {  // and the rebased mode's kernels
+      fl->reb = true;
+      st = tune();
+      fl->reb = false;
+    }
   }
-  if (st == OM_OK && starts_rebased(fl)) {
-    fl->reb = true;
-    st = rest();
-  }
+  fl->reb = starts_rebased(fl);
+  if (st == OM_OK) st = rest();
+  if (st == OM_OK && fl->rr && !fl->reb && cudaMemsetAsync(fl->rr, 0, sizeof(float) * ns->pitch, s) != cudaSuccess)
+    st = fail(OM_ECUDA, "om_flow_create: memset failed");
   if (st == OM_OK) {
     double o[4];
     st = flow_observe_any(fl, o, s);  // prev <- u_x of the rest state
@@ -894,6 +898,7 @@ extern "C" om_status om_flow_create(const om_nodeset* ns, const om_flow_params* 
 extern "C" om_status om_flow_step(om_flow* fl, int64_t nsteps, void* stream) {
   if (!fl || nsteps < 0) return fail(OM_EINVAL, "om_flow_step: bad argument");
   cudaStream_t s = as_stream(stream);
+  if (nsteps > 0) fl->observed = false;
   OM_FLOW_DISPATCH(fl, flow_steps_t, fl, nsteps, s);
 }
 
@@ -924,7 +929,8 @@ extern "C" om_status om_flow_solve(om_flow* fl, double* k_lattice, om_run_info* 
   OM_CUDA(cudaEventCreate(&e0));
   OM_CUDA(cudaEventCreate(&e1));
   double o[4];
-  OM_TRY(flow_observe_any(fl, o, s));  // reference for the first check
+  if (fl->observed) std::copy(fl->last, fl->last + 4, o);
+  else OM_TRY(flow_observe_any(fl, o, s));  // reference for the first check
   const int64_t t0 = fl->t;
   OM_CUDA(cudaEventRecord(e0, s));
   om_status rc = OM_ENOTCONVERGED;
@@ -992,6 +998,7 @@ extern "C" om_status om_flow_set_populations(om_flow* fl, const double* f_dev, v
   if (!fl || !f_dev) return fail(OM_EINVAL, "om_flow_set_populations: null pointer");
   cudaStream_t s = as_stream(stream);
   fl->t = 0;
+  fl->observed = false;
   fl->reb = starts_rebased(fl);
   auto imp = [&]() -> om_status { OM_FLOW_DISPATCH(fl, flow_import_t, fl, f_dev, s); };
   OM_TRY(imp());
@@ -1003,6 +1010,7 @@ extern "C" om_status om_flow_init_velocity(om_flow* fl, const float* ux_dev, int
                                            void* stream) {
   if (!fl || !ux_dev || stride < 1) return fail(OM_EINVAL, "om_flow_init_velocity: bad argument");
   cudaStream_t s = as_stream(stream);
+  fl->observed = false;
   fl->reb = starts_rebased(fl);
   auto init = [&]() -> om_status { OM_FLOW_DISPATCH(fl, flow_init_u_t, fl, ux_dev, stride, scale, s); };
   OM_TRY(init());

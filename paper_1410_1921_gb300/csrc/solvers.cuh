@@ -36,6 +36,10 @@ struct om_flow {
   int graph_k = 0;
   int64_t windows = 0;
   cudaStream_t cap = nullptr;
+  // prev and last are those of the present state (cleared by whatever changes it): a solve that starts
+  // from a state just observed need not observe it again
+  bool observed = false;
+  double last[4] = {0, 0, 0, 0};
 };
 
 struct om_diff {
@@ -58,6 +62,8 @@ struct om_diff {
   int graph_k = 0;
   int64_t windows = 0;
   cudaStream_t cap = nullptr;
+  bool observed = false;  // as om_flow's
+  double last[5] = {0, 0, 0, 0, 0};
 };
 
 namespace om {

@@ -135,6 +135,7 @@ extern "C" om_status om_flow_load_state(om_flow* fl, const void* host, int64_t b
     reb = h.has_cr != 0 && fl->rr != nullptr;
   }
   const bool was = fl->reb;
+  fl->observed = false;
   fl->reb = reb;
   const om_status st = load(flow_view(fl), &fl->t, host, bytes, as_stream(stream), "om_flow_load_state");
   if (st != OM_OK) fl->reb = was;
@@ -154,5 +155,6 @@ extern "C" om_status om_diff_save_state(const om_diff* df, void* host, int64_t b
 
 extern "C" om_status om_diff_load_state(om_diff* df, const void* host, int64_t bytes, void* stream) {
   if (!df) return fail(OM_EINVAL, "om_diff_load_state: null pointer");
+  df->observed = false;
   return load(diff_view(df), &df->t, host, bytes, as_stream(stream), "om_diff_load_state");
 }
