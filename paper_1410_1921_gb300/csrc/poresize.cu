@@ -33,9 +33,9 @@ __constant__ int8_t c_dir13[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1},   {1, 1
 // words (chord_lines), and a voxel's run length follows from one to three
 // words per direction by counting ones on either side of its bit
 // (chord13_kernel).  The packed lines take 13 N / 8 bytes (27 MB at 256^3: they
-// stay in L2).  The same structure: lines 205 us + rows 39 us + lengths 535 us.
+// stay in L2).  The same structure: lines 50 us + rows 39 us + lengths 535 us.
 // What bounds it now is instructions: ~26 word reads and bit scans per pore
-// voxel; the 32 byte loads per packed word in chord_lines.
+// voxel.
 //
 // Lines per direction k (e of c_dir13), position p along them:
 //   e_x = 1:         line (y0, z0), its voxel at x = 0; p = x, nx voxels, no wrap;
@@ -55,6 +55,51 @@ struct ChordLines {
 };
 
 __device__ __forceinline__ int wrap_once(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
+
+// The 32 voxels zs .. zs + 31 (periodic; nz >= 32) of row r as bits
+__device__ __forceinline__ uint32_t row_window(const uint32_t* __restrict__ rowbits, uint32_t rows, uint32_t r, int zs, int nz) {
+  const int w = zs >> 5, W = (nz + 31) >> 5;
+  const uint32_t lo = __ldg(rowbits + (uint64_t)w * rows + r);
+  const uint32_t hi = w + 1 < W ? __ldg(rowbits + (uint64_t)(w + 1) * rows + r) : 0u;
+  uint32_t b = __funnelshift_r(lo, hi, zs & 31);  // bits past nz are zero
+  if (zs + 32 > nz) b |= __ldg(rowbits + r) << (nz - zs);
+  return b;
+}
+
+// One word of 32 adjacent lines (z0 = 32 zb ..) per warp, nz >= 32, from the
+// packed rows: lane t takes the 32 voxels that step t of the 32 lines passes
+// through, one window of a row, and the warp transposes the 32 x 32 bits.
+// Byte by byte (chord_lines, left for shorter rows) the same words took
+// 202 us at 256^3, 50 us so.  blockIdx.y = direction (k = 2 excluded).
+__global__ void chord_lines_rows(ChordLines c) {
+  const int lane = threadIdx.x & 31, j = blockIdx.y, k = j < 2 ? j : j + 1;
+  const int ex = c_dir13[k][0], ey = c_dir13[k][1], ez = c_dir13[k][2];
+  const int na = ex ? c.ny : c.nx, W = ex ? c.wx : c.wy, len = ex ? c.nx : c.ny;
+  const uint32_t lines = (uint32_t)na * c.nz, rows = (uint32_t)c.nx * c.ny;
+  const uint64_t total = (uint64_t)W * na * c.wz;
+  for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < total;
+       i += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
+    const int zb = (int)(i % c.wz), a = (int)(i / c.wz % na), w = (int)(i / c.wz / na);
+    const int p = 32 * w + lane;  // position along the line
+    uint32_t b = 0;
+    if (p < len) {
+      const int x = ex ? p : a;
+      int y = ex ? a : p, z = 32 * zb;
+      if (ex && ey) y = wrap_once(y + ey * (p % c.ny), c.ny);
+      if (ez) z = wrap_once(z + ez * (p % c.nz), c.nz);
+      b = row_window(c.bits + c.off[2], rows, (uint32_t)x * c.ny + y, z, c.nz);
+    }
+    // transpose: bit t of lane s becomes bit s of lane t
+    uint32_t m = 0x0000ffffu;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1, m ^= m << s) {
+      const uint32_t o = __shfl_xor_sync(0xffffffffu, b, s);
+      b = lane & s ? (b & ~m) | ((o >> s) & m) : (b & m) | ((o << s) & ~m);
+    }
+    const int z0 = 32 * zb + lane;
+    if (z0 < c.nz) c.bits[c.off[k] + (uint64_t)w * lines + (uint32_t)a * c.nz + z0] = b;
+  }
+}
 
 // One word of one line per thread: 32 mask bytes along the line (all 32 loads
 // are independent).  blockIdx.y = direction (k = 2 excluded).
@@ -509,9 +554,14 @@ om_status chord13(const uint8_t* m, const om_domain& d, float* d_nm, int32_t* wi
     return OM_OK;
   }
   c.bits = (uint32_t*)buf.p;
-  const unsigned nb = (unsigned)std::min<uint64_t>((std::max(wx, wy) + 255) / 256, 65535);
-  chord_lines<<<dim3(nb, 12), 256, 0, s>>>(m, c);
   chord_rows<<<(unsigned)std::min<uint64_t>((wz + 7) / 8, 16 * 1216), 256, 0, s>>>(m, c);
+  if (d.nz >= 32) {
+    const uint64_t warps = (uint64_t)std::max((uint64_t)c.wx * d.ny, (uint64_t)c.wy * d.nx) * c.wz;
+    chord_lines_rows<<<dim3((unsigned)std::min<uint64_t>((warps + 7) / 8, 65535), 12), 256, 0, s>>>(c);
+  } else {
+    const unsigned nb = (unsigned)std::min<uint64_t>((std::max(wx, wy) + 255) / 256, 65535);
+    chord_lines<<<dim3(nb, 12), 256, 0, s>>>(m, c);
+  }
   chord13_kernel<<<(unsigned)std::min<uint64_t>(((uint64_t)c.N + 255) / 256, 1u << 20), 256, 0, s>>>(m, c, d.dx_nm, sq2, sq3,
                                                                                                  d_nm, witness);
   OM_CUDA(cudaGetLastError());
