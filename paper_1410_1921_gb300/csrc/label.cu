@@ -141,6 +141,14 @@ __global__ void row_pack(const uint8_t* mask, int64_t rows, int nz, int W, uint3
   }
 }
 
+__global__ void row_pack16(const uint8_t* mask, int64_t words, int nz, int W, uint32_t* bits) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / W;
+    const int w = (int)(i - r * W);
+    bits[i] = pack_word(mask + r * nz + 32 * w, min(32, nz - 32 * w));
+  }
+}
+
 // first voxel of the run that holds voxel z of a row
 __device__ __forceinline__ int run_head(const uint32_t* row, int z) {
   int w = z >> 5;
@@ -321,7 +329,8 @@ om_status label_impl(const uint8_t* mask_dev, const om_domain& d, int* labels_de
   const Rows q{bits, d.nx, d.ny, d.nz, W};
   const unsigned warps = (unsigned)std::min<int64_t>((words + 7) / 8, 16 * 1216);
   const unsigned threads = (unsigned)std::min<int64_t>((words + 127) / 128, 16 * 1216);
-  row_pack<<<warps, 256, 0, s>>>(mask_dev, rows, d.nz, W, bits);
+  if (pack_aligned(mask_dev, d.nz)) row_pack16<<<threads, 128, 0, s>>>(mask_dev, words, d.nz, W, bits);
+  else row_pack<<<warps, 256, 0, s>>>(mask_dev, rows, d.nz, W, bits);
   run_init<<<threads, 128, 0, s>>>(q, words, par);
   run_link<<<threads, 128, 0, s>>>(q, words, par);
   run_flatten<<<threads, 128, 0, s>>>(q, words, par);

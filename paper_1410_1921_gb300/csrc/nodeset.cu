@@ -32,6 +32,16 @@ __global__ void ns_bits(const uint8_t* nodes, int nz, int W, int64_t words, uint
   }
 }
 
+__global__ void ns_bits16(const uint8_t* nodes, int nz, int W, int64_t words, uint32_t* bits, uint32_t* cnt) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < words; k += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t c = k / W;
+    const int w = (int)(k - c * W);
+    const uint32_t b = pack_word(nodes + c * nz + 32 * w, min(32, nz - 32 * w));
+    bits[k] = b;
+    cnt[k] = __popc(b);
+  }
+}
+
 // node number of voxel z of the column whose first word is k0, or kNoNode
 __device__ __forceinline__ uint32_t ns_node(const uint32_t* bits, const uint32_t* rank, int64_t k0, int z) {
   const int64_t k = k0 + (z >> 5);
@@ -169,7 +179,9 @@ extern "C" om_status om_nodeset_create(const uint8_t* nodes_dev, om_domain d, vo
   uint32_t* rank = carve<uint32_t>(tmp.p, &at, nw);
   OM_CUDA(cudaMemsetAsync(total, 0, 2 * sizeof(uint64_t), s));
   const unsigned warps = (unsigned)std::min<int64_t>((nw + 7) / 8, 16 * 1216);
-  ns_bits<<<warps, 256, 0, s>>>(nodes_dev, d.nz, W, nw, bits, cnt);
+  const unsigned threads = (unsigned)std::min<int64_t>((nw + 127) / 128, 16 * 1216);
+  if (pack_aligned(nodes_dev, d.nz)) ns_bits16<<<threads, 128, 0, s>>>(nodes_dev, d.nz, W, nw, bits, cnt);
+  else ns_bits<<<warps, 256, 0, s>>>(nodes_dev, d.nz, W, nw, bits, cnt);
   ns_wrap_links<<<152, 256, 0, s>>>(nodes_dev, d.nx, d.ny, d.nz, (unsigned long long*)(total + 1));
   OM_CUDA(cudaGetLastError());
   OM_TRY(exclusive_scan_u32(cnt, rank, nw, total, s));

@@ -142,6 +142,14 @@ __global__ void chord_rows(const uint8_t* __restrict__ m, ChordLines c) {
   }
 }
 
+__global__ void chord_rows16(const uint8_t* __restrict__ m, ChordLines c) {
+  const uint32_t rows = (uint32_t)c.nx * c.ny, total = rows * (uint32_t)c.wz;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const uint32_t r = i / (uint32_t)c.wz, w = i - r * (uint32_t)c.wz;
+    c.bits[c.off[2] + (uint64_t)w * rows + r] = pack_word(m + (uint64_t)r * c.nz + 32 * w, min(32, c.nz - 32 * (int)w));
+  }
+}
+
 // Pore voxels that follow position p of line l, along the line (UP) or
 // against it; `stride` words lie between consecutive words of the line.  A
 // looping line goes on at its neighbour segment (next(l, UP)) and the count
@@ -554,7 +562,8 @@ om_status chord13(const uint8_t* m, const om_domain& d, float* d_nm, int32_t* wi
     return OM_OK;
   }
   c.bits = (uint32_t*)buf.p;
-  chord_rows<<<(unsigned)std::min<uint64_t>((wz + 7) / 8, 16 * 1216), 256, 0, s>>>(m, c);
+  if (pack_aligned(m, d.nz)) chord_rows16<<<(unsigned)std::min<uint64_t>((wz + 127) / 128, 16 * 1216), 128, 0, s>>>(m, c);
+  else chord_rows<<<(unsigned)std::min<uint64_t>((wz + 7) / 8, 16 * 1216), 256, 0, s>>>(m, c);
   if (d.nz >= 32) {
     const uint64_t warps = (uint64_t)std::max((uint64_t)c.wx * d.ny, (uint64_t)c.wy * d.nx) * c.wz;
     chord_lines_rows<<<dim3((unsigned)std::min<uint64_t>((warps + 7) / 8, 65535), 12), 256, 0, s>>>(c);
