@@ -33,7 +33,7 @@ __constant__ int8_t c_dir13[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1},   {1, 1
 // words (chord_lines), and a voxel's run length follows from one to three
 // words per direction by counting ones on either side of its bit
 // (chord13_kernel).  The packed lines take 13 N / 8 bytes (27 MB at 256^3: they
-// stay in L2).  The same structure: lines 50 us + rows 39 us + lengths 535 us.
+// stay in L2).  The same structure: lines 50 us + rows 6 us + lengths 535 us.
 // What bounds it now is instructions: ~26 word reads and bit scans per pore
 // voxel.
 //

@@ -133,7 +133,6 @@ om_status exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint6
 // ------------------------------------------------------------------ reductions
 // one block: thread t sums its share of the blocks' partials for every value,
 // the warps reduce them together and one more warp step adds the warps' sums
-//
 constexpr int kMaxVals = 8;
 __global__ void __launch_bounds__(1024) finalize_partials(const double* partials, int nblk, int nval, double* out) {
   __shared__ double sm[kMaxVals][32];
