@@ -523,13 +523,23 @@ om_status conv_tc(const om_unet* U, const bf16* x1, int c1, int ld1, int o1, con
     a.nw = N, a.npart = N / np;
     a.tx = (g.W + kTcTx - 1) / kTcTx, a.ty = (g.H + kTcTy - 1) / kTcTy;
     a.err = U->tc_err.p;
-    a.nhalo = nch + 1;
-    while (a.nhalo < kZmMaxHalo && zm_smem(a.nhalo + 1, nch, np) <= kSmem) ++a.nhalo;
-    a.nacc = std::min(kZmMaxRing, 512 / np);
-    const size_t smem = zm_smem(a.nhalo, nch, np);
-    // one CTA per SM; each part's CTAs share the planes of all columns
+    // CTAs per SM: as many, up to kZmPerSm, as leave each its weights, two planes more than it works
+    // on, a ring of at least 5 accumulators in an equal power of two of TMEM columns, and a run of 8
+    // planes or more.  Each part's CTAs share the planes of all columns.
     const int64_t planes = (int64_t)g.B * a.ty * a.tx * g.D;
-    const unsigned grid = (unsigned)(a.npart * std::min<int64_t>(planes, std::max(1, sms / a.npart)));
+    int per = kZmPerSm;
+    size_t room = 0;
+    int cols = 0;
+    for (;; --per) {
+      room = per == 1 ? kSmem : 228 * 1024 / per - 1024 - 1280;
+      cols = per == 1 ? 512 : (per == 2 ? 256 : 128);
+      if (per == 1 || (zm_smem(nch + 2, nch, np) <= room && cols / np >= 5 && planes * a.npart >= 8ll * per * sms)) break;
+    }
+    a.nhalo = nch + 1;
+    while (a.nhalo < kZmMaxHalo && zm_smem(a.nhalo + 1, nch, np) <= room) ++a.nhalo;
+    a.nacc = std::min(kZmMaxRing, cols / np);
+    const size_t smem = zm_smem(a.nhalo, nch, np);
+    const unsigned grid = (unsigned)(a.npart * std::min<int64_t>(planes, std::max(1, per * sms / a.npart)));
     auto k = nch == 1 ? (c1 <= 16 ? conv3d_tc_zm<1, 1> : conv3d_tc_zm<1, 2>) : (nch == 2 ? conv3d_tc_zm<2, 2> : conv3d_tc_zm<3, 2>);
     OM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k<<<grid, kZmThreads, smem, s>>>(m1, m2, mw, a);

@@ -355,7 +355,10 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ 
 // per tile: 20 % tensor-pipe activity).  Measured (4 x 64^3; K in, N out channels): 16 -> 32 from
 // 110 to 50 us, 32 -> 32 110 to 65, 96 -> 32 (then on conv3d_tc) 448 to 160, 64 -> 64 at 32^3 51 to 33.
 // What is left above the MMAs' own ~56 clocks each is the issuing warp's work between planes
-// (~1200 clocks: waits, commits, ring bookkeeping).
+// (~1200 clocks: waits, commits, ring bookkeeping); where the weights are few enough, two or three
+// CTAs on an SM, each with its part of the TMEM, overlap one's bookkeeping with another's MMAs (a
+// forward pass at 128^3 with 16-32-64 channels from 881 to 731 us, with two CTAs 746; a training
+// step of 4 x 64^3 with 32-64-128 channels from 2256 to 2177).
 //
 // The accumulators form a ring of R planes in TMEM: input plane z adds to planes z - 1, z, z + 1
 // (two MMAs where the ring wraps), plane z - 1 is then complete and drained by warps 2-5 (bias,
@@ -368,6 +371,7 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ 
 // columns laid end to end; a share that starts inside a column reads up to two planes more than it
 // puts out.  Waits are bounded as in conv3d_tc.
 constexpr int kZmThreads = 192;
+constexpr int kZmPerSm = 3;  // CTAs per SM where the weights leave room
 constexpr int kZmMaxRing = 32, kZmMaxHalo = 12;
 constexpr uint32_t kZmBox = (uint32_t)(kTcHx * kTcHy) * 64u;      // 11520 bytes
 constexpr uint32_t kZmBuf = (kZmBox + 1023u) / 1024u * 1024u;     // 12288

@@ -75,3 +75,10 @@ def test_gradients_of_the_fused_passes(om, ch, shape, out_ch):
     net.forward(x.cuda(), y)
     ry = R.forward(R.unflatten(0.5 * flat.cpu().double(), 2, out_ch, ch), x.double(), 2, out_ch, ch, round_bf16=True)
     assert (y.cpu().double() - ry).abs().max().item() <= 2e-2 * ry.abs().max().item()
+
+
+@pytest.mark.parametrize("ch,shape", [((16,), (1, 457, 17, 33)), ((32,), (2, 130, 17, 65))])
+def test_planes_shared_multiprocessor(om, ch, shape):
+    """Enough planes that three (16 channels) or two (32) blocks share a multiprocessor, with shares that start
+    inside a column and tiles cut at the far edges; same bounds."""
+    test_planes_match_reference(om, ch, shape)
