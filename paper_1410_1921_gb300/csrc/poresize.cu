@@ -33,7 +33,8 @@ __constant__ int8_t c_dir13[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1},   {1, 1
 // words (chord_lines), and a voxel's run length follows from one to three
 // words per direction by counting ones on either side of its bit
 // (chord13_kernel).  The packed lines take 13 N / 8 bytes (27 MB at 256^3: they
-// stay in L2).  The same structure: lines 50 us + rows 6 us + lengths 535 us.
+// stay in L2).  The same structure: lines 50 us + rows 6 us + lengths 343 us (535 with a
+// thread per voxel of the box).
 // What bounds it now is instructions: ~26 word reads and bit scans per pore
 // voxel.
 //
@@ -197,18 +198,39 @@ __device__ __forceinline__ float chord_mean(uint32_t s0, uint32_t s1, uint32_t s
   return (float)__dmul_rn(quo, dx);
 }
 
-__global__ void __launch_bounds__(256) chord13_kernel(const uint8_t* __restrict__ m, ChordLines c, double dx, double sq2,
-                                                      double sq3, float* d_nm, int32_t* witness) {
+// One block lists the pores of 256 * per consecutive voxels and then gives each
+// thread one of the list at a time: a warp of 32 voxels in a row is part solid
+// nearly everywhere, and its solid lanes would wait for the others' counts.
+constexpr int kChordPer = 8;
+
+__global__ void __launch_bounds__(256) chord13_kernel(const uint8_t* __restrict__ m, ChordLines c, int per, double dx,
+                                                      double sq2, double sq3, float* d_nm, int32_t* witness) {
+  __shared__ uint16_t list[256 * kChordPer];
+  __shared__ int count;
   const uint32_t nz = (uint32_t)c.nz, ny = (uint32_t)c.ny;
   const uint32_t plane = ny * nz, xz = (uint32_t)c.nx * nz, rows = (uint32_t)c.nx * ny;
-  for (uint64_t vv = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; vv < c.N; vv += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t v = (uint32_t)vv;
-    if (!m[v]) {
+  const uint64_t base = (uint64_t)blockIdx.x * (256 * per);
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) count = 0;
+  __syncthreads();
+  for (int i = 0; i < per; ++i) {
+    const int o = 256 * i + (int)threadIdx.x;
+    const uint64_t v = base + o;
+    const bool pore = v < c.N && m[v];
+    if (v < c.N && !pore) {
       d_nm[v] = 0.f;
       if (witness)
         for (int k = 0; k < 13; ++k) witness[(int64_t)k * c.N + v] = 0;
-      continue;
     }
+    const unsigned who = __ballot_sync(0xffffffffu, pore);
+    int at = 0;
+    if (lane == 0 && who) at = atomicAdd(&count, __popc(who));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (pore) list[at + __popc(who & ((1u << lane) - 1u))] = (uint16_t)o;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < count; i += 256) {
+    const uint32_t v = (uint32_t)(base + list[i]);
     const uint32_t row = v / nz;
     const int z = (int)(v - row * nz), x = (int)(row / ny), y = (int)(row - (uint32_t)x * ny);
     const int xy = (int)((uint32_t)x % ny), xzm = (int)((uint32_t)x % nz), yz = (int)((uint32_t)y % nz);
@@ -571,8 +593,10 @@ om_status chord13(const uint8_t* m, const om_domain& d, float* d_nm, int32_t* wi
     const unsigned nb = (unsigned)std::min<uint64_t>((std::max(wx, wy) + 255) / 256, 65535);
     chord_lines<<<dim3(nb, 12), 256, 0, s>>>(m, c);
   }
-  chord13_kernel<<<(unsigned)std::min<uint64_t>(((uint64_t)c.N + 255) / 256, 1u << 20), 256, 0, s>>>(m, c, d.dx_nm, sq2, sq3,
-                                                                                                 d_nm, witness);
+  // voxels per thread: up to kChordPer while the blocks still fill the chip (152 SMs x 8 blocks)
+  const int per = (int)std::min<uint64_t>(kChordPer, std::max<uint64_t>(1, c.N / (256u * 152 * 8)));
+  const uint64_t span = 256u * (uint64_t)per;
+  chord13_kernel<<<(unsigned)((c.N + span - 1) / span), 256, 0, s>>>(m, c, per, d.dx_nm, sq2, sq3, d_nm, witness);
   OM_CUDA(cudaGetLastError());
   return OM_OK;
 }

@@ -33,3 +33,14 @@ def test_inscribed_bricks(orc, om, shape, p):
     d, r2 = om.om_local_pore_diameter(mask, om.domain(shape, 1.5), om.OM_PORE_MIS, witness=True)
     assert rc == 0 and np.array_equal(r2, r2_o)
     assert np.array_equal(d, d_o)
+
+
+@pytest.mark.parametrize("shape", [(90, 85, 83), (140, 137, 131)])
+def test_chord13_listed_voxels(orc, om, shape):
+    """Boxes where a block lists the pores of two and of eight voxels a thread, the last block cut short."""
+    mask = S.random_mask(shape, 0.6, 13)
+    mask[: shape[0] // 3] = 0  # blocks without a pore
+    d_o, w_o = orc.chord13(mask, 1.5, counts=True)
+    d, w = om.om_local_pore_diameter(mask, om.domain(shape, 1.5), om.OM_PORE_CHORD13, witness=True)
+    assert np.array_equal(w, w_o)
+    assert np.array_equal(d, d_o)
