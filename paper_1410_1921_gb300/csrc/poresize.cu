@@ -400,10 +400,10 @@ __global__ void edt_x(const uint8_t* __restrict__ m, const int* __restrict__ h, 
 // target brick, two voxels a lane: it lists the bricks around it whose
 // largest ball reaches the target brick and exceeds the smallest radius its
 // voxels already have, and scans them from the largest on, until the next
-// one's largest ball is no larger than what every voxel has.  The ball that
-// holds a voxel is usually among the first few: 4.79 ms -> 0.30 ms, bound by
-// the instructions of the lists and scans (r2 and the brick maxima sit in
-// L1/L2).
+// one's largest ball is no larger than what every voxel has or will get from a
+// brick that lies within its own largest ball.  The ball that holds a voxel is
+// usually among the first few: 4.79 ms -> 0.28 ms, bound by the instructions of
+// the lists and scans (r2 and the brick maxima sit in L1/L2).
 constexpr int kBrick = 4;
 
 __global__ void brick_max(const int* __restrict__ r2, int nx, int ny, int nz, int nbx, int nby, int nbz, int* top) {
@@ -430,6 +430,13 @@ __device__ __forceinline__ int brick_gap(int a, int b, int n, bool periodic) {
   const int up = b - a1, down = a - b1;  // one of them positive
   const int direct = max(up, down);
   return periodic ? min(direct, n - (max(a1, b1) - min(a, b))) : direct;
+}
+
+// an upper bound of the largest distance along the line between voxels of the two intervals
+__device__ __forceinline__ int brick_far(int a, int b, int n, bool periodic) {
+  const int a1 = min(a + kBrick, n) - 1, b1 = min(b + kBrick, n) - 1;
+  const int direct = max(a1 - b, b1 - a);
+  return periodic ? min(direct, n - max(max(b - a1, a - b1), 0)) : direct;
 }
 
 constexpr int kMisWarps = 4;   // warps per block
@@ -468,30 +475,59 @@ __global__ void __launch_bounds__(32 * kMisWarps) mis_gather(const uint8_t* __re
     };
     unsigned low = least();
     if (low != 0xffffffffu) {
+      // radii that every voxel of the target has for certain: the largest ball of a brick when even
+      // the farthest pair of voxels lies within it.  First from the bricks next to the target.
+      unsigned sure = 0;
+      auto certain = [&](int qx, int qy, int qz, int t) {
+        const int fx = brick_far(bx * kBrick, qx * kBrick, nx, false);
+        const int fy = brick_far(by * kBrick, qy * kBrick, ny, true);
+        const int fz = brick_far(bz * kBrick, qz * kBrick, nz, true);
+        return fx * fx + fy * fy + fz * fz < t ? (unsigned)t : 0u;
+      };
+      if (lane < 27) {
+        const int qx = min(max(bx + lane / 9 - 1, 0), nbx - 1);
+        int qy = by + lane / 3 % 3 - 1, qz = bz + lane % 3 - 1;
+        qy = qy < 0 ? nby - 1 : (qy == nby ? 0 : qy);
+        qz = qz < 0 ? nbz - 1 : (qz == nbz ? 0 : qz);
+        sure = certain(qx, qy, qz, top[((uint32_t)qx * nby + qy) * nbz + qz]);
+      }
+      sure = __reduce_max_sync(0xffffffffu, sure);
+      if (sure > low) low = sure - 1;
       // candidate bricks: K either side in x; in y and z one more, since the
       // last brick of a line may be narrower, or all of the line once
       const int x0 = max(0, bx - K), cx = min(nbx - 1, bx + K) - x0 + 1;
       const int cy = min(nby, 2 * K + 3), cz = min(nbz, 2 * K + 3);
-      const int y0 = by - K - 1, z0 = bz - K - 1;
+      const int y0 = ((by - K - 1) % nby + nby) % nby, z0 = ((bz - K - 1) % nbz + nbz) % nbz;
       const uint32_t total = (uint32_t)cx * cy * cz;
+      // a lane's candidate (jx, jy, jz), moved on by 32 with carries instead of divisions
+      int jz = lane % cz, jy = lane / cz % cy, jx = lane / cz / cy;
+      const int sz = 32 % cz, sy = 32 / cz % cy, sx = 32 / cz / cy;
       uint32_t next = 0;
       while (next < total) {
         int cnt = 0;
         for (; next < total && cnt <= kMisList - 32; next += 32) {  // list bricks that can matter
-          const uint32_t j = next + lane;
           int t = 0;
-          uint32_t at = 0;
-          if (j < total) {
-            const int jz = (int)(j % cz), jy = (int)(j / cz % cy), jx = (int)(j / cz / cy);
-            const int qx = x0 + jx, qy = ((y0 + jy) % nby + nby) % nby, qz = ((z0 + jz) % nbz + nbz) % nbz;
-            at = ((uint32_t)qx * nby + qy) * nbz + qz;
-            t = top[at];
-            if (t > 0) {
-              const int gx = brick_gap(bx * kBrick, qx * kBrick, nx, false);
-              const int gy = brick_gap(by * kBrick, qy * kBrick, ny, true);
-              const int gz = brick_gap(bz * kBrick, qz * kBrick, nz, true);
-              if (gx * gx + gy * gy + gz * gz >= t) t = 0;
-            }
+          const int qx = x0 + jx;
+          int qy = y0 + jy, qz = z0 + jz;
+          qy -= qy >= nby ? nby : 0;
+          qz -= qz >= nbz ? nbz : 0;
+          const uint32_t at = ((uint32_t)qx * nby + qy) * nbz + qz;
+          if (next + lane < total) t = top[at];
+          jz += sz;
+          const bool c0 = jz >= cz;
+          jz -= c0 ? cz : 0;
+          jy += sy + c0;
+          const bool c1 = jy >= cy;
+          jy -= c1 ? cy : 0;
+          jx += sx + c1;
+          if (!__any_sync(0xffffffffu, t > (int)low)) continue;
+          const int gx = brick_gap(bx * kBrick, qx * kBrick, nx, false);
+          const int gy = brick_gap(by * kBrick, qy * kBrick, ny, true);
+          const int gz = brick_gap(bz * kBrick, qz * kBrick, nz, true);
+          if (gx * gx + gy * gy + gz * gz >= t) t = 0;
+          if (__any_sync(0xffffffffu, t > (int)low)) {
+            sure = __reduce_max_sync(0xffffffffu, t > (int)low ? max(sure, certain(qx, qy, qz, t)) : sure);
+            if (sure > low) low = sure - 1;
           }
           const bool keep = t > (int)low;
           const unsigned who = __ballot_sync(0xffffffffu, keep);
@@ -544,7 +580,7 @@ __global__ void __launch_bounds__(32 * kMisWarps) mis_gather(const uint8_t* __re
               }
             }
           }
-          low = least();
+          low = max(least(), low);
           __syncwarp();
         }
         __syncwarp();

@@ -44,3 +44,15 @@ def test_chord13_listed_voxels(orc, om, shape):
     d, w = om.om_local_pore_diameter(mask, om.domain(shape, 1.5), om.OM_PORE_CHORD13, witness=True)
     assert np.array_equal(w, w_o)
     assert np.array_equal(d, d_o)
+
+
+@pytest.mark.parametrize("shape", [(32, 16, 11), (40, 9, 15), (13, 22, 20)])
+@pytest.mark.parametrize("solids", [1, 5])
+def test_inscribed_large_balls(orc, om, shape, solids):
+    """Balls larger than several bricks, and wider than the box is in y and z."""
+    mask = np.ones(shape, np.uint8)
+    mask.flat[np.random.default_rng(solids).choice(mask.size, solids, replace=False)] = 0
+    rc, d_o, r2_o = orc.mis(mask, 1.5)
+    d, r2 = om.om_local_pore_diameter(mask, om.domain(shape, 1.5), om.OM_PORE_MIS, witness=True)
+    assert rc == 0 and np.array_equal(r2, r2_o)
+    assert np.array_equal(d, d_o)
