@@ -357,8 +357,8 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ 
 // What is left above the MMAs' own ~56 clocks each is the issuing warp's work between planes
 // (~1200 clocks: waits, commits, ring bookkeeping); where the weights are few enough, two or three
 // CTAs on an SM, each with its part of the TMEM, overlap one's bookkeeping with another's MMAs (a
-// forward pass at 128^3 with 16-32-64 channels from 881 to 731 us, with two CTAs 746; a training
-// step of 4 x 64^3 with 32-64-128 channels from 2256 to 2177).
+// forward pass at 128 x 120 x 136 with 16-32-64-128 channels from 881 to 731 us, with two CTAs 746;
+// a training step of 4 x 64^3 with 32-64-128 channels from 2256 to 2177).
 //
 // The accumulators form a ring of R planes in TMEM: input plane z adds to planes z - 1, z, z + 1
 // (two MMAs where the ring wraps), plane z - 1 is then complete and drained by warps 2-5 (bias,
