@@ -38,7 +38,7 @@ namespace om {
 // offsets parked in shared memory (diff_node_parked in diff_core.cuh), from
 // the records, even steps as variant 5.  5.76 M nodes, odd + even: FP32 D3Q19
 // 457 us in variant 6, 363 in 9; D3Q7 139 us, 134.  Without records 6-9 run
-// as 5.
+// as 5, and 9 as 6 where its 32-bit offsets do not reach (diff_odd_variant).
 constexpr int kDiffVariants = 10;
 
 template <class T, class L, bool ODD, int MINB>
@@ -334,6 +334,7 @@ constexpr int kDiffMinBlocks = L::Q == 7 ? 8 : 4;
 template <class T, class L, bool ODD>
 void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const DiffArgs<T, L>& a) {
   constexpr int M = kDiffMinBlocks<L>;
+  if (ODD) variant = diff_odd_variant(variant, L::Q, a.rec7 != nullptr, a.q[1] - a.q[0]);
   switch (variant) {
     case 1: launch_after(diff_sweep<T, L, ODD, M>, nb, 256, s, a); break;
     case 2: {
@@ -354,7 +355,7 @@ void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const DiffArgs<T, 
     case 6:
     case 7:
     case 8:
-      if (ODD && a.rec7) {
+      if (ODD) {
         const unsigned nbr = blocks_for((int64_t)a.nf + a.nslow);
         if (variant == 6) launch_after(diff_sweep_rec<T, L, 0>, nbr, 256, s, a);
         else if (variant == 7) launch_after(diff_sweep_rec<T, L, M>, nbr, 256, s, a);
@@ -366,7 +367,7 @@ void launch_sweep_p(int variant, unsigned nb, cudaStream_t s, const DiffArgs<T, 
       }
       [[fallthrough]];
     case 9:
-      if (ODD && a.rec7) {
+      if (ODD) {
         constexpr int B = L::Q == 19 && sizeof(T) == 8 ? 4 : 6;
         launch_after(diff_sweep_parked<T, L, B>, nb, 256, s, a);
         if (a.nslow) launch_after(diff_sweep_slow<T, L>, blocks_for(a.nslow), 256, s, a);

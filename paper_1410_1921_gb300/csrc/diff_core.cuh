@@ -225,7 +225,19 @@ __device__ __forceinline__ void diff_pair_even(const DiffArgs<T, L>& a, uint32_t
 // while the node relaxes (as flow_node_parked in flow_core.cuh): neither the
 // slot addresses nor the neighbours' reference concentrations are held, the
 // references are gathered again for the stores (they hit L1).
+// The offsets are 32-bit words, so it takes pitches whose Q populations are
+// numbered below 2^32 (parked_fits): D3Q19 up to 226 M nodes; D3Q7 any box
+// within the record fields.
 constexpr int kDiffParkStride = 256;
+__host__ __device__ constexpr bool parked_fits(int q, int64_t pitch) { return q * pitch <= (int64_t)UINT32_MAX; }
+// What launch variant v (diff.cu) runs its odd steps as, for populations of q
+// arrays of `pitch` nodes: without neighbour records 6-9 are variant 5; the
+// parked form beyond its offsets is 6, the fastest form of 64-bit addresses
+// (D3Q19, FP32, 5.76 M nodes, odd + even: 457 us against 363 parked).
+constexpr int diff_odd_variant(int v, int q, bool records, int64_t pitch) {
+  if (v >= 6 && !records) return 5;
+  return v == 9 && !parked_fits(q, pitch) ? 6 : v;
+}
 template <class T, class L, bool FACES = true>
 __device__ __forceinline__ void diff_node_parked(const DiffArgs<T, L>& a, uint32_t n, int x, const uint32_t (&nb)[L::Q],
                                                  uint32_t* parked) {
