@@ -346,12 +346,14 @@ __device__ __forceinline__ double warm_concentration(double c, double clin, doub
 // Ogita & Oishi 2008; Demmel & Nguyen 2013): with |f| < 2^E, adding and
 // subtracting 1.5 2^23 q rounds f to a multiple of q, and 19 multiples of
 // at most 2^19 q add without error.  Two such parts (q1 = 2^(E - 19), q2 =
-// 2^(E - 38)) are summed exactly, and the rest, below q2 / 2 each, in plain
-// single precision, an error below 2^(E - 58); together they form an integer
+// 2^(E - 38)) are summed exactly, and the rest, 19 terms of at most q2 / 2,
+// in plain single precision, an error below 2^(E - 55); together they form an integer
 // of 63 bits that is rounded once to double (a chain of double additions
-// rounds every step to 2^-53 of its partial sum).  Values below 2^-80 are
-// treated as of that size; sums with a non-finite term, or near overflow,
-// take the chain of double additions.
+// rounds every step to 2^-53 of its partial sum).  The parts' units are
+// single-precision normal numbers for maxima from 2^-80 to 2^114: nodes whose
+// largest population lies outside (a flux that dies away ends in subnormal
+// populations, and a sum rounded to 0 there would look converged), and sums
+// with a non-finite term, take the chain of double additions.
 struct SumMassX19 {  // sum f, sum e_x f
   static constexpr int NS = 2;
   __host__ __device__ static constexpr int s(int k, int i) { return k == 0 ? 1 : q19_e(i, 0); }
@@ -394,7 +396,8 @@ __device__ __forceinline__ void wide_sums(const float (&f)[Q], double (&out)[SG:
   uint32_t m = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i) m = max(m, __float_as_uint(f[i]) & 0x7fffffffu);
-  if (m >= (241u << 23)) {  // 2^114 and above, infinities, NaN
+  // below 2^-80 and not all 0; 2^114 and above, infinities, NaN
+  if ((m < (46u << 23) && m != 0u) || m >= (241u << 23)) {
     chain_sums<SG>(f, out);
     return;
   }
