@@ -52,3 +52,20 @@ def test_diffusion_tiny_sums(om, lattice, scale):
     df.get_fields(None, jx)
     one = flux.sum(0)
     assert np.all(np.abs(jx.cpu().numpy() - one) <= 2.0 ** -24 * np.abs(one) + 2.0 ** -150 + 2.0 ** -50 * np.abs(g).max(0))
+
+
+@pytest.mark.parametrize("scale", SCALES)
+def test_flow_tiny_sums(om, scale):
+    rng = np.random.default_rng(5)
+    u = (rng.uniform(0.5, 1.0, N) * _scale(rng, scale)).astype(np.float32)
+    fl = om.Flow(_nodes(om), om.flow_params(body_force=0.0, precision=om.OM_F32, variant=0))
+    fl.init_velocity(torch.from_numpy(u).cuda())
+    ux = fl.observe()[0]
+    # each population of the equilibrium is stored to 2^-24 of itself or half of 2^-149, ten of them carry u
+    bound = (2.0 ** -24 + 2.0 ** -50) * u.astype(np.float64) * 2 + 10 * 2.0 ** -150
+    assert abs(ux - math.fsum(u.astype(np.float64))) <= math.fsum(bound)
+    v = torch.empty(3 * N, device="cuda")
+    fl.get_velocity(v)
+    v = v.cpu().numpy()
+    assert np.all(np.abs(v[:N] - u.astype(np.float64)) <= bound + 2.0 ** -24 * u + 2.0 ** -150)
+    assert not v[N:].any()
