@@ -656,6 +656,7 @@ Grid level_grid(const Grid& g, int l) { return Grid{g.B, g.D >> l, g.H >> l, g.W
 
 om_status prepare(om_unet* U, const Grid& g) {
   if (g.B == U->grid.B && g.D == U->grid.D && g.H == U->grid.H && g.W == U->grid.W) return OM_OK;
+  U->grid = Grid{0, 0, 0, 0};  // until every buffer holds g: a failed allocation has freed its predecessor
   const int L = U->L;
   for (int l = 0; l < L; ++l) {
     const int64_t V = level_grid(g, l).voxels();
