@@ -452,9 +452,9 @@ om_status tensor_map_encoder(EncodeTiledFn* out) {
 
 // 5-D map of an NDHWC activation tensor: rows of ld BF16, c channels from o,
 // zero fill; box by mode: 0 = {64 channels, 8 x, 8 y, 2 z, 1 batch} with the
-// 128-byte swizzle, and with the 64-byte swizzle 1 = the {32, 10, 18, 3, 1}
-// halo, 2 = its one-plane form {32, 10, 18, 1, 1}, 3 = the 8 x 16 tile
-// {32, 8, 16, 1, 1}, 4 = {32, 10, 16, 3, 1}, 5 = {32, 8, 18, 1, 1}
+// 128-byte swizzle, and with the 64-byte swizzle 1 = one plane of the halo
+// {32, 10, 18, 1, 1}, 2 = the 8 x 16 tile {32, 8, 16, 1, 1}, 3 = {32, 10, 16,
+// 3, 1}, 4 = {32, 8, 18, 1, 1}
 om_status activation_map(CUtensorMap* m, const bf16* x, int c, int ld, int o, const Grid& g, int mode = 0) {
   const bool halo = mode != 0;
   EncodeTiledFn enc;
@@ -463,10 +463,10 @@ om_status activation_map(CUtensorMap* m, const bf16* x, int c, int ld, int o, co
   cuuint64_t dims[5] = {(cuuint64_t)c, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.D, (cuuint64_t)g.B};
   cuuint64_t strides[4] = {row, row * g.W, row * g.W * g.H, row * g.W * g.H * g.D};
   cuuint32_t box[5] = {(cuuint32_t)kTcKc, 8, 8, 2, 1};
-  if (mode == 1 || mode == 2) box[0] = 32, box[1] = kTcHx, box[2] = kTcHy, box[3] = mode == 1 ? kTcHz : 1;
-  if (mode == 3) box[0] = 32, box[1] = kTcTx, box[2] = kTcTy, box[3] = 1;
-  if (mode == 4) box[0] = 32, box[1] = kTcHx, box[2] = kTcTy, box[3] = 3;
-  if (mode == 5) box[0] = 32, box[1] = kTcTx, box[2] = kTcTy + 2, box[3] = 1;
+  if (mode == 1) box[0] = 32, box[1] = kTcHx, box[2] = kTcHy, box[3] = 1;
+  if (mode == 2) box[0] = 32, box[1] = kTcTx, box[2] = kTcTy, box[3] = 1;
+  if (mode == 3) box[0] = 32, box[1] = kTcHx, box[2] = kTcTy, box[3] = 3;
+  if (mode == 4) box[0] = 32, box[1] = kTcTx, box[2] = kTcTy + 2, box[3] = 1;
   cuuint32_t es[5] = {1, 1, 1, 1, 1};
   const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)(x + o), dims, strides, box, es,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, halo ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
@@ -496,13 +496,13 @@ size_t tc_smem_bytes(int N) { return 1024 + (size_t)kTcStages * (kTcATile + (siz
 
 // Y (rows of ldy, channels [oy, oy + N)) = conv of concat(x1, x2) with WT[27][N][c1 + c2]
 om_status conv_tc(const om_unet* U, const bf16* x1, int c1, int ld1, int o1, const bf16* x2, int c2, int ld2, int o2,
-                  const bf16* wt, int N, const float* bias, bf16* y, int ldy, int oy, float* yf, int relu, const Grid& g,
+                  const bf16* wt, int N, const float* bias, bf16* y, int ldy, int oy, int relu, const Grid& g,
                   cudaStream_t s) {
   if (N % 16 || N < 16 || N > 256 || c1 < 8 || (c1 % 8) || (c2 % 8) || (ld1 % 8) || (o1 % 8) || (ldy % 8) || (oy % 8))
     return fail(OM_EINVAL, "U-Net: convolution shape outside the tensor-core kernel's layout");
   CUtensorMap m1, m2, mw;
   const int nch = (c1 + 31) / 32 + (c2 + 31) / 32;
-  if (nch <= 3 && !yf) {
+  if (nch <= 3) {
     // planes marched with the weights of np output channels resident (conv3d_tc_zm): equal parts of
     // N, multiples of 16, as wide as 3 np <= 256 columns and the shared memory beside nch + 1 halo
     // buffers allow
@@ -511,8 +511,8 @@ om_status conv_tc(const om_unet* U, const bf16* x1, int c1, int ld1, int o1, con
     for (int d = 5; d >= 1 && !np; --d)
       if ((N / 16) % d == 0 && zm_smem(nch + 1, nch, 16 * d) <= kSmem) np = 16 * d;
     if ((c2 > 0 && ((ld2 % 8) || (o2 % 8)))) return fail(OM_EINVAL, "U-Net: second input not 16-byte aligned");
-    OM_TRY(activation_map(&m1, x1, c1, ld1, o1, g, 2));
-    if (c2 > 0) OM_TRY(activation_map(&m2, x2, c2, ld2, o2, g, 2));
+    OM_TRY(activation_map(&m1, x1, c1, ld1, o1, g, 1));
+    if (c2 > 0) OM_TRY(activation_map(&m2, x2, c2, ld2, o2, g, 1));
     else m2 = m1;
     OM_TRY(weight_map(&mw, wt, c1 + c2, N, true, np));
     int dev = 0, sms = 0;
@@ -555,7 +555,7 @@ om_status conv_tc(const om_unet* U, const bf16* x1, int c1, int ld1, int o1, con
   }
   OM_TRY(weight_map(&mw, wt, c1 + c2, N));
   TcConvArgs a{};
-  a.c1 = c1, a.c2 = c2, a.N = N, a.bias = bias, a.y = y, a.ldy = ldy, a.oy = oy, a.yf = yf, a.relu = relu, a.g = g;
+  a.c1 = c1, a.c2 = c2, a.N = N, a.bias = bias, a.y = y, a.ldy = ldy, a.oy = oy, a.relu = relu, a.g = g;
   a.tx = (g.W + 7) / 8, a.ty = (g.H + 7) / 8, a.tz = (g.D + 1) / 2;
   a.err = U->tc_err.p;
   OM_CUDA(cudaFuncSetAttribute(conv3d_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(N)));
@@ -576,15 +576,14 @@ om_status check_tc(const om_unet* U, cudaStream_t s) {
 
 om_status conv_forward(const om_unet* U, const Conv& c, const bf16* x1, int ld1, int o1, const bf16* x2, int ld2, int o2,
                        bf16* y, const Grid& g, cudaStream_t s) {
-  return conv_tc(U, x1, c.cin1, ld1, o1, x2, c.cin2, ld2, o2, c.wt, c.cout, U->w + c.b_off, y, c.cout, 0, nullptr, 1, g,
-                 s);
+  return conv_tc(U, x1, c.cin1, ld1, o1, x2, c.cin2, ld2, o2, c.wt, c.cout, U->w + c.b_off, y, c.cout, 0, 1, g, s);
 }
 
 // dX (rows of cin1 + cin2) = data gradient of conv c for the pre-activation gradient dyp: the
 // forward convolution of dyp with the flipped, transposed weights WD[27][cin][cout]
 om_status conv_dgrad(const om_unet* U, const Conv& c, const bf16* dyp, bf16* dx, const Grid& g, cudaStream_t s) {
   const int N = c.cin1 + c.cin2;
-  return conv_tc(U, dyp, c.cout, c.cout, 0, nullptr, 0, 0, 0, c.wd, N, nullptr, dx, N, 0, nullptr, 0, g, s);
+  return conv_tc(U, dyp, c.cout, c.cout, 0, nullptr, 0, 0, 0, c.wd, N, nullptr, dx, N, 0, 0, g, s);
 }
 
 // dW += the weight gradient on tcgen05: conv3d_wgrad_tc32 for at most 32 output channels
@@ -608,10 +607,10 @@ om_status wgrad_tc(om_unet* U, const Conv& c, const bf16* x1, int ld1, int o1, c
   if (a.Nm == 32) {
     // at most 32 output channels: the swapped form (conv3d_wgrad_tc32), all 27 offsets per CTA
     CUtensorMap m1, m2, md;
-    OM_TRY(activation_map(&m1, x1, c.cin1, ld1, o1, g, 4));
-    if (c.cin2 > 0) OM_TRY(activation_map(&m2, x2, c.cin2, ld2, o2, g, 4));
+    OM_TRY(activation_map(&m1, x1, c.cin1, ld1, o1, g, 3));
+    if (c.cin2 > 0) OM_TRY(activation_map(&m2, x2, c.cin2, ld2, o2, g, 3));
     else m2 = m1;
-    OM_TRY(activation_map(&md, dyp, c.cout, c.cout, 0, g, 5));
+    OM_TRY(activation_map(&md, dyp, c.cout, c.cout, 0, g, 4));
     a.nstage = (int)std::min<size_t>(4, (227 * 1024 - 2048) / kWnStage);
     const size_t smem = 1024 + (size_t)a.nstage * kWnStage + 8 * (2 * a.nstage + 1) + 16;
     const int gy = a.nch1 + nch2;
@@ -622,18 +621,16 @@ om_status wgrad_tc(om_unet* U, const Conv& c, const bf16* x1, int ld1, int o1, c
     OM_CUDA(cudaGetLastError());
     return OM_OK;
   }
-  // wider outputs: conv3d_wgrad_tc, the three (dz, dy) pairs of one dz per CTA
-  a.npair = 3;
-  const int hmode = 2;
+  // wider outputs: conv3d_wgrad_tc, one dz per CTA
   CUtensorMap m1, m2, md;
-  OM_TRY(activation_map(&m1, x1, c.cin1, ld1, o1, g, hmode));
-  if (c.cin2 > 0) OM_TRY(activation_map(&m2, x2, c.cin2, ld2, o2, g, hmode));
+  OM_TRY(activation_map(&m1, x1, c.cin1, ld1, o1, g, 1));
+  if (c.cin2 > 0) OM_TRY(activation_map(&m2, x2, c.cin2, ld2, o2, g, 1));
   else m2 = m1;
-  OM_TRY(activation_map(&md, dyp, c.cout, c.cout, 0, g, 3));
-  const size_t stage = wg_stage_bytes(a.npair, a.Nm);
+  OM_TRY(activation_map(&md, dyp, c.cout, c.cout, 0, g, 2));
+  const size_t stage = wg_stage_bytes(a.Nm);
   a.nstage = (int)std::min<size_t>(4, (227 * 1024 - 2048) / stage);
   const size_t smem = 1024 + (size_t)a.nstage * stage + 8 * (2 * a.nstage + 1) + 16;
-  const int gy = (a.nch1 + nch2) * (9 / a.npair) * a.npart;
+  const int gy = (a.nch1 + nch2) * 3 * a.npart;
   const int64_t ntiles = (int64_t)g.B * g.D * a.ty * a.tx;
   // one CTA per SM fits (shared memory); at most one wave, or the last CTAs run as a second
   const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntiles, sms / gy));

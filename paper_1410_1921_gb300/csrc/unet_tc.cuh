@@ -63,8 +63,7 @@ constexpr uint32_t kTcATile = kTcM * kTcKc * 2;  // 16 KB
 constexpr unsigned long long kTcSpin = 1ull << 26;  // try_wait rounds before giving up
 // the plane-marching form's and the weight gradient's tile (8 x 16 voxels at one z) and its halo box
 constexpr int kTcTx = 8, kTcTy = 16;
-constexpr int kTcHx = kTcTx + 2, kTcHy = kTcTy + 2, kTcHz = 3;
-constexpr int kTcHRows = kTcHx * kTcHy * kTcHz;  // 540 rows
+constexpr int kTcHx = kTcTx + 2, kTcHy = kTcTy + 2;
 
 struct TcConvArgs {
   int c1, c2;         // channels of the two inputs (c2 = 0: one input)
@@ -72,7 +71,6 @@ struct TcConvArgs {
   const float* bias;  // [N] or null
   bf16* y;            // output rows of ldy elements, channels [oy, oy + N)
   int ldy, oy;
-  float* yf;          // optional FP32 copy, rows of N
   int relu;
   Grid g;
   int tx, ty, tz;     // tiles along x, y, z (8, 8, 2 voxels each; the plane-marching form: 8, 16)
@@ -319,22 +317,15 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_tc(const __grid_constant__ 
         f[i] = __uint_as_float(q[i]) + (a.bias ? a.bias[c0 + i] : 0.f);
         if (a.relu) f[i] = fmaxf(f[i], 0.f);
       }
-      if (a.y) {
-        uint32_t p[8];
+      uint32_t p[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
-          p[i] = *reinterpret_cast<const uint32_t*>(&h);
-        }
-        uint4* dst = reinterpret_cast<uint4*>(a.y + v * a.ldy + a.oy + c0);
-        dst[0] = make_uint4(p[0], p[1], p[2], p[3]);
-        dst[1] = make_uint4(p[4], p[5], p[6], p[7]);
+      for (int i = 0; i < 8; ++i) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+        p[i] = *reinterpret_cast<const uint32_t*>(&h);
       }
-      if (a.yf) {
-        float4* dst = reinterpret_cast<float4*>(a.yf + v * a.N + c0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) dst[i] = make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
-      }
+      uint4* dst = reinterpret_cast<uint4*>(a.y + v * a.ldy + a.oy + c0);
+      dst[0] = make_uint4(p[0], p[1], p[2], p[3]);
+      dst[1] = make_uint4(p[4], p[5], p[6], p[7]);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -676,17 +667,16 @@ __global__ void __launch_bounds__(kZmThreads) conv3d_tc_zm(const __grid_constant
 // one MMA's 128 rows of D are the channels of the offsets dx = -1, 0, +1 (and
 // a fourth, discarded).  A K-group of 8 voxels is one x row of the tile (10
 // halo rows apart in A, 8 in B); one K = 16 MMA covers two y rows.  A CTA
-// takes one 32-channel chunk of the input, a group of (dz, dy) pairs (all
-// nine when 9 x N columns fit TMEM; the host launches it with the three of
-// one dz, for more than 32 output channels) and up to 128 output channels, keeps one TMEM accumulator per pair over every gridDim.x-th
-// tile and adds them to dW with FP32 atomics (four columns each) at the end.
+// takes one 32-channel chunk of the input, one dz with its three dy and up
+// to 128 output channels, keeps one TMEM accumulator per dy over every
+// gridDim.x-th tile and adds them to dW with FP32 atomics (four columns each)
+// at the end.  It serves more than 32 output channels.
 // Waits are bounded as in conv3d_tc.
 struct TcWgradArgs {
   int c1, c2;     // input channels of the two concatenated parts
   int nch1;       // 32-channel chunks of the first part
   int N, Nm;      // output channels, and the MMA's N (min(N, 128) rounded up to 32)
   int npart;      // parts of Nm output channels (N / 128 rounded up)
-  int npair;      // (dz, dy) pairs per CTA: 9, or 3 (one dz, a one-plane halo)
   int nstage;     // pipeline stages
   float* dw;      // [27][c1 + c2][N], accumulated
   Grid g;
@@ -695,14 +685,11 @@ struct TcWgradArgs {
   int* err;
 };
 
-constexpr uint32_t kTrHalo = ((uint32_t)kTcHRows * 64u + 1023u) / 1024u * 1024u;  // three planes of the halo
-constexpr uint32_t kWgPlane = (uint32_t)(kTcHx * kTcHy) * 64u;  // 11520: one z plane of the halo
-constexpr uint32_t kWgAtom = 128u * 64u;                         // 8192: 32 channels of the dY tile
+constexpr uint32_t kWgPlane = (uint32_t)(kTcHx * kTcHy) * 64u;              // 11520: one z plane of the halo
+constexpr uint32_t kWgHalo = (kWgPlane + 1023u) / 1024u * 1024u;            // 12288: its buffer
+constexpr uint32_t kWgAtom = 128u * 64u;                                     // 8192: 32 channels of the dY tile
 
-__host__ __device__ constexpr uint32_t wg_halo_bytes(int npair) { return npair == 9 ? kTrHalo : 12288u; }
-__host__ __device__ constexpr uint32_t wg_stage_bytes(int npair, int Nm) {
-  return wg_halo_bytes(npair) + (uint32_t)(Nm / 32) * kWgAtom;
-}
+__host__ __device__ constexpr uint32_t wg_stage_bytes(int Nm) { return kWgHalo + (uint32_t)(Nm / 32) * kWgAtom; }
 
 // MN-major shared-memory descriptor, 64-byte swizzle: MN atoms of 32
 // elements `lbo` bytes apart, K-groups of 8 rows (64 bytes each) `sbo` apart
@@ -720,7 +707,7 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = tc_smem_raw + (base - raw);
   const int S = a.nstage;
-  const uint32_t hbytes = wg_halo_bytes(a.npair), stage_bytes = wg_stage_bytes(a.npair, a.Nm);
+  const uint32_t stage_bytes = wg_stage_bytes(a.Nm);
   uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + (size_t)S * stage_bytes);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 1);
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8u * S, done = full0 + 16u * S;
@@ -728,19 +715,17 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
   __shared__ int n_issued, n_used;
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int ntiles = a.g.B * a.g.D * a.ty * a.tx;
-  // this CTA's input chunk and (dz, dy) group
-  const int ngroup = 9 / a.npair;
+  // this CTA's output channels, input chunk and dz (0..2 for -1..+1)
   const int part = (int)blockIdx.y % a.npart, n0 = part * a.Nm;
-  const int chunk = (int)blockIdx.y / a.npart / ngroup, grp = (int)blockIdx.y / a.npart % ngroup;
+  const int chunk = (int)blockIdx.y / a.npart / 3, dz = (int)blockIdx.y / a.npart % 3;
   const bool second = chunk >= a.nch1;
   const int ch0 = second ? (chunk - a.nch1) * 32 : chunk * 32;            // channel coordinate in its part
   const int cnt = min(32, (second ? a.c2 : a.c1) - ch0);                  // real channels of the chunk
   const int row0 = second ? a.c1 + ch0 : ch0;                             // its first row of dW
-  const int pair0 = grp * a.npair;                                        // first (dz, dy) pair: dz * 3 + dy
   const CUtensorMap* xm = second ? &xm2 : &xm1;
-  const uint32_t tx_bytes = (a.npair == 9 ? 3u : 1u) * kWgPlane + (uint32_t)(a.Nm / 32) * kWgAtom;
+  const uint32_t tx_bytes = kWgPlane + (uint32_t)(a.Nm / 32) * kWgAtom;
   uint32_t ncols = 32u;
-  while (ncols < (uint32_t)(a.npair * a.Nm)) ncols <<= 1;
+  while (ncols < (uint32_t)(3 * a.Nm)) ncols <<= 1;
   int mytiles = 0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) ++mytiles;
 
@@ -767,7 +752,7 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
   const uint32_t tmem = *tmem_slot;
 
   if (tid == 0) {
-    // producer: per tile the input halo (three planes, or plane z + dz) and the dY atoms
+    // producer: per tile the input halo's plane at dz and the dY atoms
     int i = 0;
     for (; i < mytiles; ++i) {
       const int st = i % S;
@@ -781,14 +766,14 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
       const int z0 = t % a.g.D, bb = t / a.g.D;
       const uint32_t sa = base + (uint32_t)st * stage_bytes, fb = full0 + 8u * st;
       mbar_expect_tx(fb, tx_bytes);
-      tma_load_5d(sa, xm, ch0, x0 - 1, y0 - 1, a.npair == 9 ? z0 - 1 : z0 + grp - 1, bb, fb);
+      tma_load_5d(sa, xm, ch0, x0 - 1, y0 - 1, z0 + dz - 1, bb, fb);
       for (int j = 0; j < a.Nm / 32; ++j)
-        tma_load_5d(sa + hbytes + (uint32_t)j * kWgAtom, &dym, n0 + 32 * j, x0, y0, z0, bb, fb);
+        tma_load_5d(sa + kWgHalo + (uint32_t)j * kWgAtom, &dym, n0 + 32 * j, x0, y0, z0, bb, fb);
       n_issued = i + 1;
     }
     if (i < mytiles) stop = 1;
   } else if (warp == 1) {
-    // MMA issue: per pair and two y rows, A = halo rows (plane, y + dy, x + dx) for dx = 0..3
+    // MMA issue: per dy and two y rows, A = halo rows (y + dy, x + dx) for dx = 0..3
     const uint32_t idesc = tc_idesc(kTcM, a.Nm) | (1u << 15) | (1u << 16), lead = elect_lane();
     int i = 0;
     for (; i < mytiles; ++i) {
@@ -797,12 +782,10 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
       n_used = i + 1;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t sa = base + (uint32_t)st * stage_bytes;
-      const uint64_t ad0 = mn_sw64_desc(sa, 64u, kTcHx * 64u), bd0 = mn_sw64_desc(sa + hbytes, kWgAtom, 512u);
-      for (int p = 0; p < a.npair; ++p) {
-        const int pr = pair0 + p, dz = pr / 3, dy = pr % 3;
-        const uint32_t row = (uint32_t)((a.npair == 9 ? dz * kTcHy : 0) + dy) * kTcHx;  // first halo row
-        const uint32_t acc_addr = tmem + (uint32_t)(p * a.Nm);
-        const uint32_t alo = lo32(ad0) + row * 4u;  // 64-byte rows in units of 16 bytes
+      const uint64_t ad0 = mn_sw64_desc(sa, 64u, kTcHx * 64u), bd0 = mn_sw64_desc(sa + kWgHalo, kWgAtom, 512u);
+      for (int dy = 0; dy < 3; ++dy) {
+        const uint32_t acc_addr = tmem + (uint32_t)(dy * a.Nm);
+        const uint32_t alo = lo32(ad0) + (uint32_t)(dy * kTcHx) * 4u;  // 64-byte rows in units of 16 bytes
         const uint32_t acc = i > 0 ? 1u : 0u;
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)  // two y rows: 2 halo rows of A, 1024 bytes of B
@@ -823,12 +806,12 @@ __global__ void __launch_bounds__(kTcThreads) conv3d_wgrad_tc(const __grid_const
   }
   // epilogue: warp w < 3 holds TMEM lanes 32 w .. + 31 = offset dx = w - 1, channel ch0 + lane
   if (!failed && mytiles > 0 && warp < 3) {
-    for (int p = 0; p < a.npair; ++p) {
-      const int k = (pair0 + p) * 3 + warp;
+    for (int dy = 0; dy < 3; ++dy) {
+      const int k = (dz * 3 + dy) * 3 + warp;
       float* dst = a.dw + ((int64_t)k * (a.c1 + a.c2) + row0 + lane) * a.N + n0;
       for (int c0 = 0; c0 < a.Nm && n0 + c0 < a.N; c0 += 16) {
         uint32_t q[16];
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(p * a.Nm + c0);
+        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dy * a.Nm + c0);
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
             "%14, %15}, [%16];"
