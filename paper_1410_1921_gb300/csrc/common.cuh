@@ -68,8 +68,10 @@ struct DevBuf {
 };
 
 // Stream-ordered scratch of one call: allocated and freed on the stream that
-// uses it, without the device-wide wait and the mapping of a cudaMalloc /
-// cudaFree pair (calls that follow each other on a stream reuse the memory).
+// uses it, without the device-wide wait of a cudaFree.  It comes from the
+// device's default pool, whose release threshold is 0: allocations that follow
+// each other on a stream reuse the memory until the host next waits for it,
+// where what is not in use goes back to the system.
 struct StreamBuf {
   void* p = nullptr;
   cudaStream_t s;

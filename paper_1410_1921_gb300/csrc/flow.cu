@@ -74,7 +74,8 @@ namespace om {
 //   14 the same with the neighbours from the records, the slow nodes in the
 //      same grid.  FP16 rebased storage: odd + even 324 us in variant 9,
 //      282 so.
-//   Without records (a box beyond their fields) 7-9 and 14 run as 6.
+//   Without records (a box beyond their fields) 7-12 run their odd steps as
+//   13 and 14 as 0; the even steps stay those of 6.
 // (Odd steps of two nodes per thread, a grid apart, with both lookups and
 // all 38 loads issued before either update, were measured slower than
 // variant 2: the registers they need halve the resident threads.)

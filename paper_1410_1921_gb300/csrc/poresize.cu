@@ -48,7 +48,7 @@ __constant__ int8_t c_dir13[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1},   {1, 1
 // read adjacent words; for k = 2 lines are (x, y) rows and lanes share them.
 struct ChordLines {
   int nx, ny, nz;
-  uint32_t N;            // voxels (a box of more takes the walking kernel)
+  uint32_t N;            // voxels (check_domain keeps them below 2^32 - 1)
   int wx, wy, wz;        // words per line along x, y, z
   uint32_t loop;         // voxels of a closed (0, 1, +-1) loop: lcm(ny, nz)
   uint32_t* bits;
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(256) chord13_kernel(const uint8_t* __restrict_
 }
 
 // The walking form, without scratch memory: what is left when the packed
-// lines cannot be allocated (or the box is beyond their 32-bit indices).
+// lines cannot be allocated.
 // Cells along +-e from (x,y,z), stopping at solid or the x faces; *closed is
 // set when the walk comes back to its start (an all-pore loop).
 __device__ int walk(const uint8_t* __restrict__ m, int nx, int ny, int nz, int x, int y, int z, int ex,
