@@ -313,25 +313,38 @@ __device__ __forceinline__ void flow_rebase_node(const FlowArgs<T>& a, uint32_t 
 
 // f = f_eq(rho = 1, u = (u, 0, 0)) as deviations from w_i in the even layout:
 // w_i t(e_ix) with t(0) = -1.5 u^2 and t(+-1) = +-3 u + 3 u^2, three values
-// of t and three weights, the diagonal one half the axis one: halving the
-// rounded axis value is exact in binary except among subnormals, where the
-// diagonal one is rounded from its own product.  Nine double operations a node; per population they were 7 x 19,
+// of t and three weights, the diagonal one half the axis one (exact in
+// binary, except among subnormals).  Nine double operations a node; per population they were 7 x 19,
 // and 331 us of FP64 pipe on 5.76 M nodes (173 us so, the read of u and its clamp included).
+// Where a population may be subnormal in single precision, each is rounded
+// from its own product (flow_store_eq_x_tiny).  That is a call, not a branch
+// inline: predicated, its double operations took the FP64 pipe of every node
+// (5.35 M nodes, with the observation after it: 501 us without, 562 inline, 502 so).
+template <class T>
+__device__ __noinline__ void flow_store_eq_x_tiny(T* s, uint32_t P, double u, typename Stg<T>::C up) {
+  const double q = u * u, t0 = -1.5 * q, tp = fma(3.0, q, 3.0 * u), tm = fma(3.0, q, -3.0 * u);
+#pragma unroll
+  for (int i = 0; i < 19; ++i) {
+    const double t = q19_e(i, 0) == 0 ? t0 : (q19_e(i, 0) > 0 ? tp : tm);
+    Stg<T>::st(s + (uint64_t)i * P, (typename Stg<T>::C)(q19_w(i) * t), up);
+  }
+}
+
 template <class T>
 __device__ __forceinline__ void flow_store_eq_x(const FlowArgs<T>& a, uint32_t n, double u) {
   using C = typename Stg<T>::C;
   const double q = u * u, t0 = -1.5 * q, tp = fma(3.0, q, 3.0 * u), tm = fma(3.0, q, -3.0 * u);
   const C rest = (C)(q19_w(0) * t0);
   const C ax[3] = {(C)(q19_w(1) * tm), (C)(q19_w(1) * t0), (C)(q19_w(1) * tp)};  // [e_x + 1]
-  auto diagonal = [](C v, double t) {
-    if (sizeof(C) == 4 && fabs(v) < C(0x1p-125)) return (C)(q19_w(7) * t);
-    return C(0.5) * v;
-  };
-  const C di[3] = {diagonal(ax[0], tm), diagonal(ax[1], t0), diagonal(ax[2], tp)};
+  const uint32_t hi = (uint32_t)__double2hiint(u) & 0x7fffffffu;
+  if (sizeof(C) == 4 && hi < (963u << 20) && hi != 0u) {  // 0 < |u| < 2^-60: u^2 / 12 and u / 6 may be subnormal
+    flow_store_eq_x_tiny<T>(a.s[0] + n, a.P, u, a.up);
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < 19; ++i) {
-    const int k = q19_e(i, 0) + 1;
-    Stg<T>::st(a.s[i] + n, i == 0 ? rest : (i < 7 ? ax[k] : di[k]), a.up);
+    const C v = ax[q19_e(i, 0) + 1];
+    Stg<T>::st(a.s[i] + n, i == 0 ? rest : (i < 7 ? v : C(0.5) * v), a.up);
   }
 }
 
